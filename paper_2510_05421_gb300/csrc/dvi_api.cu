@@ -276,7 +276,8 @@ size_t layout(dvi_ctx* c, char* base) {
     const size_t nqkv = static_cast<size_t>(c->Hq + 2 * c->Hkv) * c->hd;
     a.xr = reinterpret_cast<float*>(take(sizeof(float) * 2 * B * d));
     a.qkv = reinterpret_cast<float*>(take(sizeof(float) * B * nqkv));
-    a.att = reinterpret_cast<float*>(take(sizeof(float) * B * c->Hq * a.P * (c->hd + 2)));
+    a.att = reinterpret_cast<float*>(take(sizeof(float) * B * c->Hq * a.P * c->hd));
+    a.att_ml = reinterpret_cast<float*>(take(sizeof(float) * B * c->Hq * a.P * 2));
     a.ao = reinterpret_cast<float*>(take(sizeof(float) * B * d));
     a.hbuf = reinterpret_cast<float*>(take(sizeof(float) * B * c->F));
     a.y = reinterpret_cast<float*>(take(sizeof(float) * B * d));

@@ -292,7 +292,7 @@ struct MkArgs {
   int mode;
   int B, k, d, Hq, Hkv, hd, F, V, max_len, K, Kv, r;
   const CUtensorMap* wmaps;   // [k][7] (wq, wk, wv, wo, wg, wu, wd), then W^S: 16 tiles of 8 rows x 64
-  int P;                 // attention position splits per (sequence, KV head)
+  int P;                 // attention position ranges per (sequence, KV head), at most (<= 16)
   int n_stages;          // weight ring stages of 16 KB
   int rows_max;          // output rows of one CTA in any phase
   int n_bound;           // completion counters (the abort flag follows them)
@@ -310,7 +310,8 @@ struct MkArgs {
   // scratch
   float* xr;             // [2][B][d] residual stream (double buffered)
   float* qkv;            // [B][(H_q + 2 H_kv) hd] projections before RoPE
-  float* att;            // [B][H_q][P][hd + 2] attention partials (max, sum, o)
+  float* att;            // [B][H_q][P][hd] attention partials: o
+  float* att_ml;         // [B][H_q][P][2] their (max, sum)
   float* ao;             // [B][d] output projection
   float* hbuf;           // [B][F] SwiGLU
   float* y;              // [B][d] down projection

@@ -28,9 +28,9 @@
 // its result does not depend on the CTA count or on how many decode rows
 // share the launch.
 //
-// The attention of a decode row at position pos splits [0, pos] into P equal
-// ranges (a function of pos only, so a draft pass and a greedy AR step at the
-// same position reduce in the same order).  The ring streams a range in
+// The attention of a decode row at position pos splits [0, pos] into ranges
+// of whole ring chunks (a function of pos only, so a draft pass and a greedy
+// AR step at the same position reduce in the same order).  The ring streams a range in
 // chunks of 8192 / hd cached positions, keys then values, each one 16 KB TMA
 // box; positions written earlier in this launch and the newest one are
 // filled into the stage from global memory and from the pass's own K/V.
@@ -42,7 +42,13 @@
 namespace dvi {
 namespace {
 
-constexpr int kMkThreads = 288;      // warps 0-7 compute, warp 8 streams
+// Warps 0-7 compute, warp 8 streams (warps 9-11 complete its warpgroup).  A
+// thread is launched with 168 registers (65536 / 384); the warpgroups then
+// split the same 64512 as 2 x 128 x 232 and 128 x 40, so the compute warps
+// hold a phase's loads in flight without spilling.
+constexpr int kMkThreads = 384;
+constexpr int kMkComputeRegs = 232, kMkStreamRegs = 40;
+static_assert(256 * kMkComputeRegs + 128 * kMkStreamRegs <= kMkThreads * 168, "the launch's registers");
 constexpr int kMkCompute = 256;
 constexpr int kMkWarps = 8;
 constexpr int kMkStage = 16384;      // bytes per ring stage
@@ -162,20 +168,26 @@ struct Ring {
   uint64_t* full;
   uint64_t* empty;
   int ns;
-  uint32_t it;   // stages consumed so far (the same sequence as the producer's)
+  int slot;       // the next stage's slot and parity (the same sequence as the producer's)
+  uint32_t par;
+  __device__ __forceinline__ void next() {
+    if (++slot == ns) {
+      slot = 0;
+      par ^= 1u;
+    }
+  }
 };
 
 // Compute side: wait for the next stage's bytes.
 __device__ __forceinline__ const uint8_t* ring_acquire(Ring& r, int* status, bool& ok) {
-  const int s = static_cast<int>(r.it % r.ns);
-  if (!mbar_wait(&r.full[s], (r.it / r.ns) & 1u, status)) ok = false;
-  return r.base + static_cast<size_t>(s) * kMkStage;
+  if (!mbar_wait(&r.full[r.slot], r.par, status)) ok = false;
+  return r.base + static_cast<size_t>(r.slot) * kMkStage;
 }
 // Compute side: the warp is done with the stage (one arrival per warp).
 __device__ __forceinline__ void ring_release(Ring& r) {
   __syncwarp();
-  if ((threadIdx.x & 31) == 0) mbar_arrive(&r.empty[r.it % r.ns]);
-  ++r.it;
+  if ((threadIdx.x & 31) == 0) mbar_arrive(&r.empty[r.slot]);
+  r.next();
 }
 
 // ------------------------------------------------------------------ boundaries
@@ -377,11 +389,26 @@ __device__ __forceinline__ const CUtensorMap* qkv_group(const MkArgs& a, int l, 
   return m + 2;
 }
 
-// Attention unit (sequence b, KV head kvh, range p of P) of CTA c, if any,
-// and its position range [r0, r1) of [0, pos] at pass j.
+// Ranges that [0, pos] is split into (a function of pos only): about
+// kMkUnitChunks ring chunks of 8192 / hd positions each, at most P.  A range
+// more costs every CTA a partial row per query head in the O phase's combine
+// (16 of them at the 1B shape: 133 KB, 8 us; 5: 42 KB), a chunk more costs
+// its unit about 0.4 us.
+// Draft phase of the 1B workload (5 passes of 8 layers, 512 positions) 2.08
+// -> 1.41 ms and of the 7B one (5 x 2, 1024) 1.14 -> 1.06 ms, with the O
+// phase's combine and the compute warps' registers.
+constexpr int kMkUnitChunks = 2;
+__device__ __forceinline__ int att_chunks(int pos, int hd) { return pos / (kMkStageElems / hd) + 1; }
+__device__ __forceinline__ int att_parts(const MkArgs& a, int pos) {
+  return min(a.P, (att_chunks(pos, a.hd) + kMkUnitChunks - 1) / kMkUnitChunks);
+}
+
+// Attention unit (sequence b, KV head kvh, range p of the parts) of CTA c, if
+// any, and its position range [r0, r1) of [0, pos] at pass j (whole chunks
+// but for the last).
 struct AttUnit {
   bool on;
-  int b, kvh, p, pos, n_b, r0, r1;
+  int b, kvh, p, np, pos, n_b, r0, r1;
 };
 __device__ __forceinline__ AttUnit att_unit(const MkArgs& a, int j, int c) {
   AttUnit u;
@@ -392,7 +419,12 @@ __device__ __forceinline__ AttUnit att_unit(const MkArgs& a, int j, int c) {
   u.p = c % a.P;
   u.n_b = a.lens[u.b];
   u.pos = u.n_b + j;
-  part_range(u.pos + 1, u.p, a.P, u.r0, u.r1);
+  u.np = att_parts(a, u.pos);
+  u.on = u.p < u.np;
+  const int cp = kMkStageElems / a.hd;
+  part_range(att_chunks(u.pos, a.hd), u.p, u.np, u.r0, u.r1);
+  u.r0 *= cp;
+  u.r1 = min(u.r1 * cp, u.pos + 1);
   return u;
 }
 // Positions of the chunk [c0, c0 + cn) of a unit that the ring streams: those
@@ -416,10 +448,10 @@ template <int HD>
 __device__ void mk_producer(const MkArgs& a, Ring& r, int c, int n) {
   constexpr int CP = kMkStageElems / HD;
   const uint64_t pol = l2_evict_first_policy();
-  uint32_t it = 0;
+  uint32_t it = 0;   // stages issued
   auto take = [&](int& s) -> bool {
-    s = static_cast<int>(it % r.ns);
-    return mbar_wait_abort(&r.empty[s], ((it / r.ns) & 1u) ^ 1u, a);
+    s = r.slot;
+    return mbar_wait_abort(&r.empty[s], r.par ^ 1u, a);
   };
   // one 8-row group of a K-column matrix: its 1024-column chunks, each one
   // box of 16 tiles of 8 rows x 64 (tiles past K and rows past the matrix
@@ -431,6 +463,7 @@ __device__ void mk_producer(const MkArgs& a, Ring& r, int c, int n) {
       if (!take(s)) return false;
       mbar_arrive_expect_tx(&r.full[s], static_cast<uint32_t>(kMkStage));
       tma_load_3d(r.base + static_cast<size_t>(s) * kMkStage, map, 0, y, kc * (kMkChunk / 64), &r.full[s], pol);
+      r.next();
       ++it;
     }
     return true;
@@ -449,6 +482,7 @@ __device__ void mk_producer(const MkArgs& a, Ring& r, int c, int n) {
     if (!take(s)) return false;
     mbar_arrive_expect_tx(&r.full[s], static_cast<uint32_t>(kMkStage));
     tma_load_3d(r.base + static_cast<size_t>(s) * kMkStage, map, 0, row, 0, &r.full[s], kv_pol);
+    r.next();
     ++it;
     return true;
   };
@@ -581,8 +615,7 @@ namespace {
 
 // The normed input of a projection over d columns in one pass (d <= 4096):
 // x = xa + xb (or the embedding of tok), stored to xr_out by `writer`; the
-// per-128-feature sums of squares (tsum) and 1/rms (rstd); the A planes of
-// x * rstd * g.  Thread tid takes the column pairs tid + 256 e, whose loads
+// per-128-feature sums of squares and 1/rms; the A planes of x * rstd * g.  Thread tid takes the column pairs tid + 256 e, whose loads
 // (x and gain) are all issued before any is used; a warp's 32 pairs are half
 // a 128-column tile, so the tile sums are two warp sums (hs[m][tile][half]).
 constexpr int kMkPairs = 8;   // column pairs per thread: d <= 512 * kMkPairs
@@ -590,7 +623,7 @@ template <int M>
 __device__ __forceinline__ void mk_norm_pack(const MkArgs& a, const float* __restrict__ xa,
                                              const float* __restrict__ xb, const int* tok, float* xr_out,
                                              bool writer, const float* __restrict__ g, uint32_t* xw, int plane,
-                                             float* tsum, float* rstd, float* hs) {
+                                             float* hs) {
   const int d = a.d, np = d / 2, nt = d / 128, pw = plane / 2;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float2 x[M][kMkPairs], gv[kMkPairs];
@@ -629,23 +662,21 @@ __device__ __forceinline__ void mk_norm_pack(const MkArgs& a, const float* __res
     }
   }
   cbar();
-  if (tid < M) {
-    float s = 0.f;
-    for (int t = 0; t < nt; ++t) {
-      const float ts = hs[(tid * nt + t) * 2] + hs[(tid * nt + t) * 2 + 1];
-      tsum[tid * nt + t] = ts;
-      s += ts;
-    }
-    rstd[tid] = rsqrtf(s / static_cast<float>(d) + a.eps);
+  // every warp sums the row's tiles itself, one a lane (nt <= 32): no
+  // serial chain over the tiles and no second barrier
+  float rs[M];
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const float2 t = lane < nt ? reinterpret_cast<const float2*>(hs)[m * nt + lane] : make_float2(0.f, 0.f);
+    rs[m] = rsqrtf(warp_sum(t.x + t.y) / static_cast<float>(d) + a.eps);
   }
-  cbar();
 #pragma unroll
   for (int e = 0; e < kMkPairs; ++e) {
     const int p = tid + e * kMkCompute;
     if (p < np) {
 #pragma unroll
       for (int m = 0; m < M; ++m) {
-        const float r = rstd[m];
+        const float r = rs[m];
         uint32_t hi, lo;
         split_bf16x2(x[m][e].x * r * gv[e].x, x[m][e].y * r * gv[e].y, hi, lo);
         xw[(2 * m) * pw + p] = hi;
@@ -778,7 +809,7 @@ __device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& rin
   }
   cbar();
   // the newest position into the cache (the unit whose range ends at pos)
-  if (u.p == a.P - 1) {
+  if (u.p == u.np - 1) {
     if (pos_ok) {
       const size_t row = kv_row(a, l, u.b, u.kvh, u.pos) * HD;
       for (int dim = tid; dim < HD; dim += kMkCompute) {
@@ -938,7 +969,6 @@ __device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& rin
     }
   }
   cbar();
-  const size_t stride = HD + 2;
   for (int i = tid; i < G * HD; i += kMkCompute) {
     const int gg = i / HD, dd = i % HD;
     float m = -INFINITY;
@@ -954,12 +984,9 @@ __device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& rin
         if (dd == 0) sum = fmaf(e, wml[(w * G + gg) * 2 + 1], sum);
       }
     }
-    float* dst = a.att + ((static_cast<size_t>(u.b) * a.Hq + u.kvh * G + gg) * a.P + u.p) * stride;
-    dst[2 + dd] = v;
-    if (dd == 0) {
-      dst[0] = m;
-      dst[1] = sum;
-    }
+    const size_t part = (static_cast<size_t>(u.b) * a.Hq + u.kvh * G + gg) * a.P + u.p;
+    a.att[part * HD + dd] = v;
+    if (dd == 0) *reinterpret_cast<float2*>(a.att_ml + 2 * part) = make_float2(m, sum);
   }
   return true;
 }
@@ -980,74 +1007,92 @@ __device__ __forceinline__ bool mk_attention_any(const MkArgs& a, int l, const A
   }
 }
 
-// The O phase's input: for every row and query head the P partials merged
-// (weights exp2(m_p - max) / sum) and packed straight into the A planes
-// (column pairs of H_q hd; four pairs per thread at a time, all their
-// partials' loads issued together).
+// The O phase's input: for every row and query head the partials of its
+// ranges merged (weights exp2(m_p - max) / sum) and packed straight into the
+// A planes.  Latency-bound (every CTA rebuilds the row from L2 before its
+// first product), so the loads are issued together: half a warp per (row,
+// head) takes the head's (max, sum) pairs, one range a lane, and finishes
+// them by shuffles; then four columns per thread and step (float4), four
+// ranges' loads in flight for two steps at a time, each range added in order.
+// With the weights summed range by range and one column pair a thread this
+// phase's prologue took 15.7 us of a 47 us layer at the 1B shape (16 ranges)
+// and 7.1 us of 89 at the 7B shape (4 ranges).
 template <int HD, int M>
-__device__ __forceinline__ void mk_att_combine(const MkArgs& a, uint32_t* xw, int plane, float* wts) {
-  const int K = a.Hq * HD, P = a.P, np = K / 2, pw = plane / 2;
-  const size_t stride = HD + 2;
-  for (int i = threadIdx.x; i < a.B * a.Hq; i += kMkCompute) {
-    const float* base = a.att + static_cast<size_t>(i) * P * stride;
-    float mx = -INFINITY;
-    for (int p = 0; p < P; ++p) mx = fmaxf(mx, __ldcg(base + p * stride));
-    float sum = 0.f;
-    for (int p = 0; p < P; ++p) sum += __ldcg(base + p * stride + 1) * exp2f(__ldcg(base + p * stride) - mx);
-    const float inv = 1.f / sum;
-    for (int p = 0; p < P; ++p) wts[i * P + p] = exp2f(__ldcg(base + p * stride) - mx) * inv;
+__device__ __forceinline__ void mk_att_combine(const MkArgs& a, const int (&np)[M], uint32_t* xw, int plane,
+                                               float* wts) {
+  const int K = a.Hq * HD, P = a.P, nq4 = K / 4, pw = plane / 2;
+  const int lane = threadIdx.x & 31, sub = lane & 15;
+  for (int i0 = (threadIdx.x >> 5) * 2; i0 < M * a.Hq; i0 += 2 * kMkWarps) {
+    const int i = i0 + (lane >> 4);
+    float2 ml = make_float2(-INFINITY, 0.f);
+    if (i < M * a.Hq) {
+      const int n = M == 1 || i < a.Hq ? np[0] : np[M - 1];
+      if (sub < n) ml = __ldcg(reinterpret_cast<const float2*>(a.att_ml) + static_cast<size_t>(i) * P + sub);
+    }
+    float mx = ml.x;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const float e = ml.x == -INFINITY ? 0.f : exp2f(ml.x - mx);
+    float sum = e * ml.y;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (i < M * a.Hq && sub < P) wts[i * P + sub] = e / sum;
   }
   cbar();
-  for (int q0 = threadIdx.x; q0 < np; q0 += 4 * kMkCompute) {
 #pragma unroll
-    for (int m = 0; m < M; ++m) {
-      float2 s[4];
+  for (int m = 0; m < M; ++m) {
+    for (int q0 = threadIdx.x; q0 < nq4; q0 += 2 * kMkCompute) {
+      float4 s[2];
+      const float* src[2];
+      const float* w[2];
+      bool on[2];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) s[u] = make_float2(0.f, 0.f);
-      for (int p = 0; p < P; ++p) {
-        float2 v[4];
+      for (int u = 0; u < 2; ++u) {
+        const int q = q0 + u * kMkCompute;
+        on[u] = q < nq4;
+        const int h = on[u] ? (4 * q) / HD : 0;
+        src[u] = a.att + (static_cast<size_t>(m) * a.Hq + h) * P * HD + (on[u] ? (4 * q) % HD : 0);
+        w[u] = wts + (m * a.Hq + h) * P;
+        s[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      for (int p0 = 0; p0 < np[m]; p0 += 4) {
+        float4 v[2][4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int q = q0 + u * kMkCompute;
-          v[u] = make_float2(0.f, 0.f);
-          if (q < np)
-            v[u] = __ldcg(reinterpret_cast<const float2*>(
-                a.att + ((static_cast<size_t>(m) * a.Hq + (2 * q) / HD) * P + p) * stride + 2 + (2 * q) % HD));
-        }
+        for (int u = 0; u < 2; ++u)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int q = q0 + u * kMkCompute;
-          if (q < np) {
-            const float wgt = wts[(m * a.Hq + (2 * q) / HD) * P + p];
-            s[u].x = fmaf(v[u].x, wgt, s[u].x);
-            s[u].y = fmaf(v[u].y, wgt, s[u].y);
-          }
-        }
+          for (int p = 0; p < 4; ++p)
+            if (on[u] && p0 + p < np[m])
+              v[u][p] = __ldcg(reinterpret_cast<const float4*>(src[u] + static_cast<size_t>(p0 + p) * HD));
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int p = 0; p < 4; ++p)
+            if (on[u] && p0 + p < np[m]) {
+              const float x = w[u][p0 + p];
+              s[u].x = fmaf(v[u][p].x, x, s[u].x);
+              s[u].y = fmaf(v[u][p].y, x, s[u].y);
+              s[u].z = fmaf(v[u][p].z, x, s[u].z);
+              s[u].w = fmaf(v[u][p].w, x, s[u].w);
+            }
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int q = q0 + u * kMkCompute;
-        if (q < np) {
-          uint32_t hi, lo;
-          split_bf16x2(s[u].x, s[u].y, hi, lo);
-          xw[(2 * m) * pw + q] = hi;
-          xw[(2 * m + 1) * pw + q] = lo;
-        }
+      for (int u = 0; u < 2; ++u) {
+        if (!on[u]) continue;
+        const int q = 2 * (q0 + u * kMkCompute);
+        uint2 hi, lo;
+        split_bf16x2(s[u].x, s[u].y, hi.x, lo.x);
+        split_bf16x2(s[u].z, s[u].w, hi.y, lo.y);
+        *reinterpret_cast<uint2*>(xw + (2 * m) * pw + q) = hi;
+        *reinterpret_cast<uint2*>(xw + (2 * m + 1) * pw + q) = lo;
       }
     }
   }
   const int nw = mk_chunks(K) * kMkChunk / 2;
-  for (int w = np + threadIdx.x; w < nw; w += kMkCompute)
+  for (int w = K / 2 + threadIdx.x; w < nw; w += kMkCompute)
 #pragma unroll
     for (int q = 0; q < 2 * M; ++q) xw[q * pw + w] = 0u;
   cbar();
 }
-
-}  // namespace
-}  // namespace dvi
-
-namespace dvi {
-namespace {
 
 }  // namespace
 }  // namespace dvi
@@ -1091,6 +1136,9 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
   for (int j = 0; j < npass; ++j) {
     const bool head = a.mode == MK_DRAFT && j < K;
     const AttUnit u = att_unit(a, j, c);
+    int np[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) np[m] = att_parts(a, a.lens[m] + j);
     for (int l = 0; l < a.k; ++l) {
       const MkLayerW& w = a.layer[l];
       // ---------------- QKV
@@ -1116,8 +1164,7 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
         cbar();
       }
       if (fused) {
-        mk_norm_pack<M>(a, xr[cur], a.y, l == 0 ? tok : nullptr, xr[cur ^ 1], c == 0, w.g_attn, xw, plane, tsum, rstd,
-                        hs);
+        mk_norm_pack<M>(a, xr[cur], a.y, l == 0 ? tok : nullptr, xr[cur ^ 1], c == 0, w.g_attn, xw, plane, hs);
       } else {
         if (l == 0) mk_residual(a, act, nullptr, nullptr, tok, xr[cur ^ 1], c == 0);
         else mk_residual(a, act, xr[cur], a.y, nullptr, xr[cur ^ 1], c == 0);
@@ -1144,7 +1191,7 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
       bw = bn++;
       // ---------------- O
       if (!mk_wait(a, bw, flag_s)) return;
-      mk_att_combine<HD, M>(a, xw, plane, reinterpret_cast<float*>(att_sm));
+      mk_att_combine<HD, M>(a, np, xw, plane, reinterpret_cast<float*>(att_sm));
       if (!gemv_groups<M>(ring, nq, o0, o1, xa, plane, wacc, rows_max, a.status)) {
         mk_abort(a);
         return;
@@ -1157,7 +1204,7 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
       // ---------------- gate / up
       if (!mk_wait(a, bw, flag_s)) return;
       if (fused) {
-        mk_norm_pack<M>(a, xr[cur], a.ao, nullptr, xr[cur ^ 1], c == 0, w.g_ffn, xw, plane, tsum, rstd, hs);
+        mk_norm_pack<M>(a, xr[cur], a.ao, nullptr, xr[cur ^ 1], c == 0, w.g_ffn, xw, plane, hs);
       } else {
         mk_residual(a, act, xr[cur], a.ao, nullptr, xr[cur ^ 1], c == 0);
         mk_rms(a, act, tsum, rstd);
@@ -1347,7 +1394,8 @@ __global__ void __launch_bounds__(kMkThreads, 1) mk_kernel(const __grid_constant
   ring.full = reinterpret_cast<uint64_t*>(sm + L.bars);
   ring.empty = ring.full + a.n_stages;
   ring.ns = a.n_stages;
-  ring.it = 0;
+  ring.slot = 0;
+  ring.par = 0u;
   const int tid = threadIdx.x;
   if (tid == 0) {
     for (int s = 0; s < a.n_stages; ++s) {
@@ -1362,9 +1410,11 @@ __global__ void __launch_bounds__(kMkThreads, 1) mk_kernel(const __grid_constant
   if (tid < 4) reinterpret_cast<uint32_t*>(sm + L.xw)[M * mk_plane(a) + tid] = 0u;
   __syncthreads();
   if (tid >= kMkCompute) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMkStreamRegs));
     if (tid == kMkCompute) mk_producer<HD>(a, ring, blockIdx.x, gridDim.x);
     return;
   }
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kMkComputeRegs));
   mk_compute<M, HD>(a, ring, L, sm);
 }
 
@@ -1395,6 +1445,14 @@ void mk_attrs() {
 int mk_ctas_per_sm(const MkArgs& a) {
   if (a.B < 1 || a.B > kMkMaxRows || (a.hd != 64 && a.hd != 128)) return 0;
   mk_attrs();
+  // the compute warps' register increase draws on what the block was
+  // launched with: never run the kernel if that is less than the split needs
+  cudaFuncAttributes fa{};
+  if (cudaFuncGetAttributes(&fa, mk_pick(a)) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (fa.numRegs * kMkThreads < 256 * kMkComputeRegs + 128 * kMkStreamRegs) return 0;
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, mk_pick(a), kMkThreads, mk_smem_bytes(a, a.n_stages)) !=
       cudaSuccess) {

@@ -139,6 +139,16 @@ def test_two_ragged_sequences_lossless_and_oracle():
     _check_first_step(w, W, P, max_seq_len=cap)
 
 
+@pytest.mark.parametrize("n", [62, 126, 127, 128, 640, 2100])
+def test_attention_ranges(n):
+    """Contexts around the edges of the attention's position ranges (chunks of
+    64 positions at head_dim 128, two chunks a range, at most 16 ranges): one
+    partial range up to 16 ranges of several chunks."""
+    w = _bf16_case().with_(prompt_len=(n, n), gen_tokens=12)
+    W, P, _ = _lossless(w)
+    _check_first_step(w, W, P)
+
+
 def test_1b_full_size_lossless_and_every_step():
     w = workload("1b").with_(gen_tokens=24)
     W = make_weights(w)
