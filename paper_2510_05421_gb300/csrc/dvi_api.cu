@@ -631,6 +631,7 @@ AttnArgs attn_args(dvi_ctx* ctx, int l, const Pass& ps) {
   // the positions: one CTA walks its rows' whole prefix
   t.n_splits_max = dec_cluster ? (ps.pf ? 1 : ctx->dec_nsplits) : ctx->attn_nsplits;
   t.prefill = ps.pf && dec_cluster ? 1 : 0;
+  t.n_sms = ctx->n_sms;
   t.part = ctx->attn_part;
   t.counters = ctx->attn_ctr;
   t.status = ctx->status;

@@ -156,6 +156,7 @@ struct AttnArgs {
   const CUtensorMap* kmap;           // bf16 decode: the K / V caches as [rows][hd] (box 64 x 64)
   const CUtensorMap* vmap;
   int prefill;                       // a prompt pass (bf16, GQA group <= 8): the prefill attention kernel
+  int n_sms;
   const int* dep_wait; int dep_count; int* dep_signal;   // chained launch (as ProjArgs; bf16 decode kernel)
 };
 // CTAs of the attention launch for these arguments.
@@ -167,6 +168,8 @@ bool make_kv_map(CUtensorMap* map, const void* cache, long long rows, int hd);
 size_t attn_partial_floats(const AttnArgs& a);
 int attn_counters(const AttnArgs& a);
 cudaError_t launch_attn(const AttnArgs& a, cudaStream_t s);
+// The prefill attention kernel (attn_pf.cu; a.prefill set).
+cudaError_t launch_attn_pf(const AttnArgs& a, cudaStream_t s);
 
 // ---- small kernels (misc.cu)
 struct EmbedArgs {

@@ -81,3 +81,34 @@ def test_prefill_chunk_size_does_not_change_the_cache():
         assert np.array_equal(k, outs[0][0])
         assert np.array_equal(v, outs[0][1])
         assert first == outs[0][2]
+
+
+# (query heads, KV heads, head_dim, prompt): one partial tile of 128 query
+# vectors, tile and chunk edges, GQA groups that do not divide 128, and enough
+# (row, head) pairs that a CTA takes two tiles
+TILES = [(4, 4, 64, 1), (4, 4, 64, 127), (4, 4, 64, 129), (6, 2, 64, 130), (16, 2, 64, 257), (4, 2, 128, 128),
+         (32, 32, 64, 700), (20, 20, 128, 1025)]
+
+
+@pytest.mark.parametrize("hq,hkv,hd,n", TILES)
+def test_attention_tiles(hq, hkv, hd, n):
+    """Layer 2's K/V rows, which carry layer 1's attention output, against the
+    oracle within two bf16 steps of the largest entry (2^-7 relative), and
+    bit-identical whichever rows share a pass (chunks of 48 rows)."""
+    from paper_2510_05421_gb300 import DeviceWeights
+    from workloads import tiny_shape
+    w = workload("tiny").with_(dtype="bf16", prompt_len=(n, n), split_k=1,
+                               shape=tiny_shape(n_layers=2, n_heads=hq, n_kv_heads=hkv, head_dim=hd))
+    W = make_weights(w)
+    P = make_prompts(w)
+    dw = DeviceWeights.from_host(W, "bf16")
+    k, v, first = _prefill(w, dw, P, 0)
+    m = OracleModel(rounded_weights(W), w.shape, w.lora_gamma, dtype=np.float64, kv_dtype="bf16")
+    cache = m.new_cache(n + 1)
+    oracle_prefill(m, cache, P[0])
+    for got, ref in ((k, cache.k), (v, cache.v)):
+        for l in range(2):
+            r = ref[l, :n].transpose(1, 0, 2)
+            assert np.abs(got[l] - r).max() <= 2.0 ** -7 * np.abs(r).max(), l
+    k2, v2, first2 = _prefill(w, dw, P, 48)
+    assert np.array_equal(k, k2) and np.array_equal(v, v2) and first == first2
