@@ -87,71 +87,78 @@ __device__ __forceinline__ void pf_row_pos(const ProjArgs& p, int n, int& seq, i
   pos = p.lens[seq] + p.pos_off + n % p.rows_per_seq;
 }
 
+// A row's values read ahead of the accumulator: the residual's first steps
+// (O, down) or the rotations of the first 16 dims (QKV).
+constexpr int kResAhead = 4;
+using Ahead = float4[kResAhead][4];
+
 // QKV: RoPE (rotate-half pairs dim and dim + hd/2 of one head, both in the
 // tile since sections and heads are 128-aligned), q rows in f32, k and v
-// rows into the cache at the row's position.
-__device__ __forceinline__ void pf_epi_qkv(const ProjArgs& p, uint32_t acc, int nt, int n, bool live, float rstd) {
+// rows into the cache at the row's position.  16 dims at a time over every
+// head of the tile, so a rotation is read once, one step ahead of its use.
+__device__ __forceinline__ void pf_load_rope(const ProjArgs& p, int pos, int j, Ahead& ahead) {
+  const float4* r = reinterpret_cast<const float4*>(p.rope + static_cast<size_t>(pos) * (p.head_dim >> 1) + j);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) ahead[e >> 2][e & 3] = __ldg(r + e);
+}
+__device__ __forceinline__ void pf_epi_qkv(const ProjArgs& p, uint32_t acc, int nt, int n, int seq, int pos, bool st,
+                                           float rstd, Ahead& ahead) {
   const int hd = p.head_dim, half = hd >> 1;
-  int seq = 0, pos = 0;
-  if (live) pf_row_pos(p, n, seq, pos);
-  const bool pos_ok = pos >= 0 && pos < p.max_len;
-  if (live && !pos_ok) flag_status(p.status, DVI_DEV_KV_FULL);
-  const bool st = live && pos_ok;
-  for (int h = 0; h < 2; ++h) {
-    const int f0 = nt * kPfN + h * kTileRows;
-    int sec, fl;
-    if (f0 < p.rows_q) { sec = 0; fl = f0; }
-    else if (f0 < p.rows_q + p.rows_k) { sec = 1; fl = f0 - p.rows_q; }
-    else if (f0 < p.rows_q + p.rows_k + p.rows_v) { sec = 2; fl = f0 - p.rows_q - p.rows_k; }
-    else break;
-    for (int hh = 0; hh < kTileRows / hd; ++hh) {
-      const int c0 = h * kTileRows + hh * hd;
-      const int head = (fl + hh * hd) / hd;
-      for (int j = 0; j < half; j += 16) {
-        float a[16], b[16];
-        tmem_ld16(acc + static_cast<uint32_t>(c0 + j), a);
-        tmem_ld16(acc + static_cast<uint32_t>(c0 + half + j), b);
-        if (!st) continue;
+  for (int j = 0; j < half; j += 16) {
+    float4 rot[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) rot[e] = ahead[e >> 2][e & 3];
+    if (st && j + 16 < half) pf_load_rope(p, pos, j + 16, ahead);
+    for (int c0 = 0; c0 < kPfN; c0 += hd) {
+      const int f0 = nt * kPfN + c0;
+      int sec, fl;
+      if (f0 < p.rows_q) { sec = 0; fl = f0; }
+      else if (f0 < p.rows_q + p.rows_k) { sec = 1; fl = f0 - p.rows_q; }
+      else if (f0 < p.rows_q + p.rows_k + p.rows_v) { sec = 2; fl = f0 - p.rows_q - p.rows_k; }
+      else break;
+      const int head = fl / hd;
+      float a[16], b[16];
+      tmem_ld16(acc + static_cast<uint32_t>(c0 + j), a);
+      tmem_ld16(acc + static_cast<uint32_t>(c0 + half + j), b);
+      if (!st) continue;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        a[e] *= rstd;
+        b[e] *= rstd;
+      }
+      if (sec < 2) {
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
-          a[e] *= rstd;
-          b[e] *= rstd;
+          const float rx = e & 1 ? rot[e >> 1].z : rot[e >> 1].x, ry = e & 1 ? rot[e >> 1].w : rot[e >> 1].y;
+          const float x1 = a[e] * rx - b[e] * ry;
+          const float x2 = b[e] * rx + a[e] * ry;
+          a[e] = x1;
+          b[e] = x2;
         }
-        if (sec < 2) {
-          const float2* cs = p.rope + static_cast<size_t>(pos) * half + j;
+      }
+      if (sec == 0) {
+        float4* q0 = reinterpret_cast<float4*>(p.q_out + static_cast<size_t>(n) * p.ld_q + head * hd + j);
+        float4* q1 = reinterpret_cast<float4*>(p.q_out + static_cast<size_t>(n) * p.ld_q + head * hd + half + j);
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const float2 r = cs[e];
-            const float x1 = a[e] * r.x - b[e] * r.y;
-            const float x2 = b[e] * r.x + a[e] * r.y;
-            a[e] = x1;
-            b[e] = x2;
-          }
+        for (int e = 0; e < 4; ++e) {
+          q0[e] = make_float4(a[4 * e], a[4 * e + 1], a[4 * e + 2], a[4 * e + 3]);
+          q1[e] = make_float4(b[4 * e], b[4 * e + 1], b[4 * e + 2], b[4 * e + 3]);
         }
-        if (sec == 0) {
-          float4* q0 = reinterpret_cast<float4*>(p.q_out + static_cast<size_t>(n) * p.ld_q + head * hd + j);
-          float4* q1 = reinterpret_cast<float4*>(p.q_out + static_cast<size_t>(n) * p.ld_q + head * hd + half + j);
+      } else {
+        __nv_bfloat16* c = static_cast<__nv_bfloat16*>(sec == 1 ? p.kc : p.vc) +
+                           ((static_cast<size_t>(seq) * p.n_kv_heads + head) * p.max_len + pos) * hd;
+        uint32_t pa[8], pb[8];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            q0[e] = make_float4(a[4 * e], a[4 * e + 1], a[4 * e + 2], a[4 * e + 3]);
-            q1[e] = make_float4(b[4 * e], b[4 * e + 1], b[4 * e + 2], b[4 * e + 3]);
-          }
-        } else {
-          __nv_bfloat16* c = static_cast<__nv_bfloat16*>(sec == 1 ? p.kc : p.vc) +
-                             ((static_cast<size_t>(seq) * p.n_kv_heads + head) * p.max_len + pos) * hd;
-          uint32_t pa[8], pb[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            pa[e] = pack_bf16x2(a[2 * e], a[2 * e + 1]);
-            pb[e] = pack_bf16x2(b[2 * e], b[2 * e + 1]);
-          }
-          uint4* c0p = reinterpret_cast<uint4*>(c + j);
-          uint4* c1p = reinterpret_cast<uint4*>(c + half + j);
-          c0p[0] = make_uint4(pa[0], pa[1], pa[2], pa[3]);
-          c0p[1] = make_uint4(pa[4], pa[5], pa[6], pa[7]);
-          c1p[0] = make_uint4(pb[0], pb[1], pb[2], pb[3]);
-          c1p[1] = make_uint4(pb[4], pb[5], pb[6], pb[7]);
+        for (int e = 0; e < 8; ++e) {
+          pa[e] = pack_bf16x2(a[2 * e], a[2 * e + 1]);
+          pb[e] = pack_bf16x2(b[2 * e], b[2 * e + 1]);
         }
+        uint4* c0p = reinterpret_cast<uint4*>(c + j);
+        uint4* c1p = reinterpret_cast<uint4*>(c + half + j);
+        c0p[0] = make_uint4(pa[0], pa[1], pa[2], pa[3]);
+        c0p[1] = make_uint4(pa[4], pa[5], pa[6], pa[7]);
+        c1p[0] = make_uint4(pb[0], pb[1], pb[2], pb[3]);
+        c1p[1] = make_uint4(pb[4], pb[5], pb[6], pb[7]);
       }
     }
   }
@@ -159,45 +166,62 @@ __device__ __forceinline__ void pf_epi_qkv(const ProjArgs& p, uint32_t acc, int 
 
 // O and down: x += y, the next norm's activation rows x * g (hi/lo), and
 // the sums of squares of the new x per 128 features (in feature order).
-__device__ __forceinline__ void pf_epi_resid(const ProjArgs& p, uint32_t acc, int nt, int n, bool live) {
-  for (int h = 0; h < 2; ++h) {
-    const int f0 = nt * kPfN + h * kTileRows;
-    if (f0 >= p.n_out) break;
-    float ssq = 0.f;
-    for (int j = 0; j < kTileRows; j += 16) {
+// The tile's residual row is read kResAhead steps of 16 features ahead of
+// its use (a step's four loads take about a microsecond, with one thread a
+// row and nothing else in flight: 16 of them in turn were a tail of 12 us).
+__device__ __forceinline__ void pf_epi_resid(const ProjArgs& p, uint32_t acc, int nt, int n, bool live,
+                                             Ahead& ahead) {
+  const int f00 = nt * kPfN;
+  const int steps = min(kPfN, p.n_out - f00) / 16;
+  float* xrow = p.x_res + static_cast<size_t>(live ? n : 0) * p.ld_res + f00;
+  float ssq = 0.f;
+#pragma unroll 1
+  for (int s0 = 0; s0 < steps; s0 += kResAhead) {
+#pragma unroll
+    for (int u = 0; u < kResAhead; ++u) {
+      const int st = s0 + u;
       float v[16];
-      tmem_ld16(acc + static_cast<uint32_t>(h * kTileRows + j), v);
-      if (!live) continue;
-      const int f = f0 + j;
-      float4* xp = reinterpret_cast<float4*>(p.x_res + static_cast<size_t>(n) * p.ld_res + f);
+      tmem_ld16(acc + static_cast<uint32_t>(st * 16), v);
       float x[16];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const float4 t = __ldcg(xp + e);
+        const float4 t = ahead[u][e];
         x[4 * e] = t.x + v[4 * e];
         x[4 * e + 1] = t.y + v[4 * e + 1];
         x[4 * e + 2] = t.z + v[4 * e + 2];
         x[4 * e + 3] = t.w + v[4 * e + 3];
       }
+      if (live) {
+        if (st + kResAhead < steps) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) xp[e] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
-#pragma unroll
-      for (int e = 0; e < 16; ++e) ssq += x[e] * x[e];
-      if (p.xg_out) {
-        const float4* g4 = reinterpret_cast<const float4*>(p.g_next + f);
-        float y[16];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float4 g = g4[e];
-          y[4 * e] = x[4 * e] * g.x;
-          y[4 * e + 1] = x[4 * e + 1] * g.y;
-          y[4 * e + 2] = x[4 * e + 2] * g.z;
-          y[4 * e + 3] = x[4 * e + 3] * g.w;
+          for (int e = 0; e < 4; ++e)
+            ahead[u][e] = __ldcg(reinterpret_cast<const float4*>(xrow + (st + kResAhead) * 16) + e);
         }
-        st_act16(static_cast<__nv_bfloat16*>(p.xg_out) + static_cast<size_t>(n) * p.ld_xg + f, p.xg_plane, y);
+        const int f = f00 + st * 16;
+        float4* xp = reinterpret_cast<float4*>(xrow + st * 16);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) xp[e] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) ssq += x[e] * x[e];
+        if (p.xg_out) {
+          const float4* g4 = reinterpret_cast<const float4*>(p.g_next + f);
+          float y[16];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float4 g = g4[e];
+            y[4 * e] = x[4 * e] * g.x;
+            y[4 * e + 1] = x[4 * e + 1] * g.y;
+            y[4 * e + 2] = x[4 * e + 2] * g.z;
+            y[4 * e + 3] = x[4 * e + 3] * g.w;
+          }
+          st_act16(static_cast<__nv_bfloat16*>(p.xg_out) + static_cast<size_t>(n) * p.ld_xg + f, p.xg_plane, y);
+        }
+        if ((st & 7) == 7) {
+          p.ss_out[static_cast<size_t>(f / kTileRows) * p.ss_out_ld + n] = ssq;
+          ssq = 0.f;
+        }
       }
     }
-    if (live) p.ss_out[static_cast<size_t>(f0 / kTileRows) * p.ss_out_ld + n] = ssq;
   }
 }
 
@@ -267,7 +291,6 @@ __global__ void __launch_bounds__(192, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  griddep_launch();
   const uint32_t tmem = *tmem_holder;
 
   if (warp == 4) {
@@ -346,6 +369,10 @@ __global__ void __launch_bounds__(192, 1)
           }
           tc_commit(&empty[s]);
         }
+        // The next kernel's CTAs may take their places once every CTA's last
+        // tile is issued: its epilogue covers their launch.  From the start
+        // they would hold SMs (this kernel's 200 KB each) while they wait.
+        if (t + static_cast<int>(gridDim.x) >= n_tiles) griddep_launch();
         // also after a failed wait, so the epilogue's wait ends and every
         // MMA issued has completed before the TMEM is freed
         tc_commit(&accf[b]);
@@ -369,12 +396,30 @@ __global__ void __launch_bounds__(192, 1)
         for (int q = 0; q < p.ss_tiles; ++q) sq += __ldcg(p.ss + static_cast<size_t>(q) * p.ss_ld + n);
         rstd = rsqrtf(sq / static_cast<float>(p.d_norm) + p.eps);
       }
+      // and what its epilogue reads first: the residual row's first steps (nt * 256
+      // + 64 <= n_out: n_out is a multiple of 128), or the row's first rotations
+      Ahead ahead;
+      int seq = 0, pos = 0;
+      bool st = live;
+      if (p.flavor == EPI_QKV && live) {
+        pf_row_pos(p, n, seq, pos);
+        st = pos >= 0 && pos < p.max_len;
+        if (!st) flag_status(p.status, DVI_DEV_KV_FULL);
+        else pf_load_rope(p, pos, 0, ahead);
+      }
+      if (p.flavor == EPI_RESID && live) {
+        const float4* x4 = reinterpret_cast<const float4*>(p.x_res + static_cast<size_t>(n) * p.ld_res + nt * kPfN);
+#pragma unroll
+        for (int u = 0; u < kResAhead; ++u)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ahead[u][e] = __ldcg(x4 + 4 * u + e);
+      }
       if (!mbar_wait(&accf[b], (j >> 1) & 1, p.status)) break;
       tc_fence_after();
       const uint32_t acc = tmem + (static_cast<uint32_t>(warp * 32) << 16) + static_cast<uint32_t>(b * kPfN);
-      if (p.flavor == EPI_QKV) pf_epi_qkv(p, acc, nt, n, live, rstd);
+      if (p.flavor == EPI_QKV) pf_epi_qkv(p, acc, nt, n, seq, pos, st, rstd, ahead);
       else if (p.flavor == EPI_GATEUP) pf_epi_gateup(p, acc, nt, n, live, rstd);
-      else pf_epi_resid(p, acc, nt, n, live);
+      else pf_epi_resid(p, acc, nt, n, live, ahead);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acce[b]);
