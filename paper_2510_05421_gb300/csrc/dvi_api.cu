@@ -43,6 +43,7 @@ struct Pass {
   void* xg;
   const CUtensorMap* xg_map;
   bool pf = false;   // a bf16 prompt pass: projections on the prefill kernel
+  int n_tokens = 0;  // of the prompt (pf)
 };
 
 struct Plan {
@@ -760,7 +761,7 @@ bool use_chain(const dvi_ctx* ctx, const Pass& ps) {
 // next layer's attention norm, or the final norm before a head).
 // A projection of a bf16 prompt pass on the prefill kernel, with the
 // activation buffer's 128-row map and the weights' 128-row maps.
-dvi_status run_proj_pf(dvi_ctx* ctx, const ProjLaunch& pl, const CUtensorMap& act, const CUtensorMap& w0,
+dvi_status run_proj_pf(dvi_ctx* ctx, const ProjLaunch& pl, int n_tokens, const CUtensorMap& act, const CUtensorMap& w0,
                        const CUtensorMap* w1 = nullptr, const CUtensorMap* w2 = nullptr) {
   ProjArgs a = pl.a;
   if (a.xg_out) a.xg_plane = act_plane(ctx, a.xg_out, a.ld_xg);
@@ -770,7 +771,7 @@ dvi_status run_proj_pf(dvi_ctx* ctx, const ProjLaunch& pl, const CUtensorMap& ac
   m.w0 = w0;
   m.w1 = w1 ? *w1 : w0;
   m.w2 = w2 ? *w2 : w0;
-  DVI_CUDA(launch_proj_pf(a, m, ctx->n_sms, ctx->stream));
+  DVI_CUDA(launch_proj_pf(a, m, n_tokens, ctx->n_sms, ctx->stream));
   ++ctx->launches;
   return DVI_OK;
 }
@@ -780,13 +781,13 @@ dvi_status run_proj_pf(dvi_ctx* ctx, const ProjLaunch& pl, const CUtensorMap& ac
 dvi_status enqueue_layer_pf(dvi_ctx* ctx, int l, const Pass& ps, const float* g_last) {
   const LayerMaps& m = ctx->maps[l];
   dvi_status st;
-  if ((st = run_proj_pf(ctx, qkv_launch(ctx, l, ps), ctx->map_pf_xg, m.qkv.m0, &m.qkv.m1, &m.qkv.m2)) != DVI_OK)
+  if ((st = run_proj_pf(ctx, qkv_launch(ctx, l, ps), ps.n_tokens, ctx->map_pf_xg, m.qkv.m0, &m.qkv.m1, &m.qkv.m2)) != DVI_OK)
     return st;
   DVI_CUDA(launch_attn(attn_args(ctx, l, ps), ctx->stream));
   ++ctx->launches;
-  if ((st = run_proj_pf(ctx, o_launch(ctx, l, ps), ctx->map_pf_attn_o, m.o.m0)) != DVI_OK) return st;
-  if ((st = run_proj_pf(ctx, gu_launch(ctx, l, ps), ctx->map_pf_xg, m.gate128, &m.up128)) != DVI_OK) return st;
-  return run_proj_pf(ctx, down_launch(ctx, l, ps, g_last), ctx->map_pf_ffn_h, m.down.m0);
+  if ((st = run_proj_pf(ctx, o_launch(ctx, l, ps), ps.n_tokens, ctx->map_pf_attn_o, m.o.m0)) != DVI_OK) return st;
+  if ((st = run_proj_pf(ctx, gu_launch(ctx, l, ps), ps.n_tokens, ctx->map_pf_xg, m.gate128, &m.up128)) != DVI_OK) return st;
+  return run_proj_pf(ctx, down_launch(ctx, l, ps, g_last), ps.n_tokens, ctx->map_pf_ffn_h, m.down.m0);
 }
 
 dvi_status enqueue_layer(dvi_ctx* ctx, int l, const Pass& ps, const float* g_last) {
@@ -1339,7 +1340,7 @@ dvi_status dvi_prefill(dvi_ctx* ctx, int seq, const int32_t* d_tokens, int n_tok
     e.status = ctx->status;
     DVI_CUDA(launch_embed(e, s));
     ctx->launches += 1;
-    Pass ps{ctx->x_pf, ctx->ss_pf, ctx->pf_rows, rows, rows, seq, 1, c0, ctx->xg_pf, &ctx->map_xg_pf, ctx->tc};
+    Pass ps{ctx->x_pf, ctx->ss_pf, ctx->pf_rows, rows, rows, seq, 1, c0, ctx->xg_pf, &ctx->map_xg_pf, ctx->tc, n_tokens};
     dvi_status rc = enqueue_layers(ctx, 0, ctx->L, ps);
     if (rc != DVI_OK) return rc;
     last_rows = rows;

@@ -110,7 +110,8 @@ bool make_act_map_box(CUtensorMap* map, const void* act, int rows, int cols, int
 struct PfMaps {
   CUtensorMap act, w0, w1, w2;
 };
-cudaError_t launch_proj_pf(const ProjArgs& a, const PfMaps& m, int n_sms, cudaStream_t s);
+// `n_tokens`: the whole prompt's length (it decides the split over K).
+cudaError_t launch_proj_pf(const ProjArgs& a, const PfMaps& m, int n_tokens, int n_sms, cudaStream_t s);
 
 // Persistent projection chain (bf16): up to kChainMax projections of one
 // pass in a single launch, each phase's output feeding the next phase's B

@@ -112,3 +112,34 @@ def test_attention_tiles(hq, hkv, hd, n):
             assert np.abs(got[l] - r).max() <= 2.0 ** -7 * np.abs(r).max(), l
     k2, v2, first2 = _prefill(w, dw, P, 48)
     assert np.array_equal(k, k2) and np.array_equal(v, v2) and first == first2
+
+
+# (d, query heads, KV heads, head_dim, d_ffn, prompt): the 1B width at 1, 2, 3
+# and 6 row tiles (QKV split 8, 4, 2 and 1 ways over K; O 8, 8, 4, 2; gate/up
+# 2, 1; down 8, 8, 4, 2), a width with head_dim 64, and a d_ffn whose last K
+# range is empty (33 K blocks over 8 ranges) and whose last tile is partial
+SPLITS = [(2048, 16, 8, 128, 5632, 17), (2048, 16, 8, 128, 5632, 129), (2048, 16, 8, 128, 5632, 300),
+          (2048, 16, 8, 128, 5632, 700), (1024, 16, 4, 64, 2816, 40), (1024, 8, 8, 128, 2088, 130)]
+
+
+@pytest.mark.parametrize("d,hq,hkv,hd,f,n", SPLITS)
+def test_short_prompts_split_over_k(d, hq, hkv, hd, f, n):
+    """Prompts whose projections split K over a cluster: the caches against the
+    oracle (as above) and bit-identical in passes of 48 rows."""
+    from paper_2510_05421_gb300 import DeviceWeights
+    from workloads import tiny_shape
+    w = workload("tiny").with_(dtype="bf16", prompt_len=(n, n), split_k=1,
+                               shape=tiny_shape(n_layers=2, d_model=d, n_heads=hq, n_kv_heads=hkv, head_dim=hd, d_ffn=f))
+    W = make_weights(w)
+    P = make_prompts(w)
+    dw = DeviceWeights.from_host(W, "bf16")
+    k, v, first = _prefill(w, dw, P, 0)
+    m = OracleModel(rounded_weights(W), w.shape, w.lora_gamma, dtype=np.float64, kv_dtype="bf16")
+    cache = m.new_cache(n + 1)
+    oracle_prefill(m, cache, P[0])
+    for got, ref in ((k, cache.k), (v, cache.v)):
+        for l in range(2):
+            r = ref[l, :n].transpose(1, 0, 2)
+            assert np.abs(got[l] - r).max() <= 2.0 ** -7 * np.abs(r).max(), l
+    k2, v2, first2 = _prefill(w, dw, P, 48)
+    assert np.array_equal(k, k2) and np.array_equal(v, v2) and first == first2
