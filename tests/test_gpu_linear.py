@@ -64,3 +64,26 @@ def test_linear_deterministic_and_row_independent(eng):
     assert torch.equal(y1, y2)
     assert torch.equal(y_one[0], y1[0])
     assert torch.equal(y_five, y1[:5])
+
+
+@pytest.mark.parametrize("n,k,m,off", [(1, 1, 1, 0), (130, 33, 3, 0), (130, 66, 5, 1), (300, 100, 4, 1),
+                                       (257, 1000, 17, 3), (64, 31, 16, 2)])
+def test_f32_any_k_and_alignment(n, k, m, off):
+    """The f32 kernel's weight blocks: K not a multiple of 4 or of the block,
+    operands at any 4-byte address (no float4 loads then), row counts on both
+    sides of the four-column variant; against a float64 matmul."""
+    from paper_2510_05421_gb300.dvi import linear_noalloc
+    g = np.random.default_rng(n + k)
+    W = g.standard_normal((n, k)).astype(np.float32)
+    X = g.standard_normal((m, k)).astype(np.float32)
+    w = torch.empty(n * k + off, device="cuda")[off:].view(n, k)
+    x = torch.empty(m * k + off, device="cuda")[off:].view(m, k)
+    w.copy_(torch.from_numpy(W))
+    x.copy_(torch.from_numpy(X))
+    y = torch.empty(m, n, device="cuda")
+    assert linear_noalloc(w, x, y) == 0
+    torch.cuda.synchronize()
+    ref = X.astype(np.float64) @ W.astype(np.float64).T
+    # K products and sums of f32: at most (K + 1) 2^-24 of sum |x||w|
+    bound = (k + 1) * 2.0 ** -24 * (np.abs(X).astype(np.float64) @ np.abs(W).astype(np.float64).T)
+    assert (np.abs(y.cpu().numpy() - ref) <= bound).all()
