@@ -153,13 +153,64 @@ __device__ __forceinline__ int take_argmax(unsigned long long* slot, int* status
   return argmax_idx(k);
 }
 
-// Embeds each sequence's next input token into the draft residual stream.
-template <typename T, int NT = kMaxTiles>
-__device__ void embed_rows(const StepState& st, const int* toks, float* red) {
-  for (int b = 0; b < st.B; ++b)
-    embed_row_block<T, NT>(static_cast<const T*>(st.embed), toks[b], st.d, st.x_dr + static_cast<size_t>(b) * st.d,
-                       st.g0, static_cast<T*>(st.xg_dr) + static_cast<size_t>(b) * st.d, st.xg_dr_plane, st.ss_dr,
-                       st.ss_dr_ld, b, red);
+// Four consecutive values (a column that is a multiple of 4); one vector load
+// where the row's address allows it.
+__device__ __forceinline__ float4 ld_row4(const float* p, bool vec) {
+  return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ float4 ld_row4(const __nv_bfloat16* p, bool vec) {
+  if (!vec) return make_float4(__bfloat162float(p[0]), __bfloat162float(p[1]), __bfloat162float(p[2]),
+                               __bfloat162float(p[3]));
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  return make_float4(bf16_lo(u.x), bf16_hi(u.x), bf16_lo(u.y), bf16_hi(u.y));
+}
+// The activation row's four values at p (hi and lo planes for bf16).
+__device__ __forceinline__ void st_act_row4(float* p, size_t, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void st_act_row4(__nv_bfloat16* p, size_t plane, float4 v) {
+  uint2 hi, lo;
+  split_bf16x2(v.x, v.y, hi.x, lo.x);
+  split_bf16x2(v.z, v.w, hi.y, lo.y);
+  *reinterpret_cast<uint2*>(p) = hi;
+  *reinterpret_cast<uint2*>(p + plane) = lo;
+}
+
+// Embeds each sequence's next input token into the draft residual stream: x,
+// x * g and the per-tile sums of squares.  A warp per eight 128-feature tiles
+// of a row, four features of each a lane, its loads in flight together;
+// `staged`: the rows in shared memory, else they come from the table.  (One row after
+// another by all 128 threads took 14 us a row: 110 of a draft head's 162 us
+// at batch 8.)
+template <typename T>
+__device__ void embed_rows(const StepState& st, const int* toks, const T* staged = nullptr) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int d = st.d, nt = d / kTileRows;
+  const bool gvec = (reinterpret_cast<uintptr_t>(st.g0) & 15u) == 0;
+  const bool svec = staged || (reinterpret_cast<uintptr_t>(st.embed) & 15u) == 0;
+  const int parts = (nt + 7) / 8;
+  for (int it = warp; it < st.B * parts; it += kFinThreads / 32) {
+    const int b = it / parts, t0 = it % parts * 8;
+    const T* src = (staged ? staged + static_cast<size_t>(b) * d
+                           : static_cast<const T*>(st.embed) + static_cast<size_t>(toks[b]) * d) + 4 * lane;
+    float* x = st.x_dr + static_cast<size_t>(b) * d + 4 * lane;
+    T* xg = static_cast<T*>(st.xg_dr) + static_cast<size_t>(b) * d + 4 * lane;
+    float4 v[8], g[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int t = min(t0 + u, nt - 1);
+      v[u] = ld_row4(src + t * kTileRows, svec);
+      g[u] = ld_row4(st.g0 + t * kTileRows + 4 * lane, gvec);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int t = t0 + u;
+      if (t >= nt) break;
+      *reinterpret_cast<float4*>(x + t * kTileRows) = v[u];
+      st_act_row4(xg + t * kTileRows, st.xg_dr_plane,
+                  make_float4(v[u].x * g[u].x, v[u].y * g[u].y, v[u].z * g[u].z, v[u].w * g[u].w));
+      const float q = warp_sum((v[u].x * v[u].x + v[u].y * v[u].y) + (v[u].z * v[u].z + v[u].w * v[u].w));
+      if (lane == 0) st.ss_dr[static_cast<size_t>(t) * st.ss_dr_ld + b] = q;
+    }
+  }
 }
 
 
@@ -208,18 +259,14 @@ __device__ void finalize_draft_body(const StepState& st, int j, const HeadPrepAr
   }
   if (!next) return;
   if (!emb_raw) {
-    embed_rows<T, NT>(st, fs.tok_s, fs.red);
+    embed_rows<T>(st, fs.tok_s);
     return;
   }
   cp_async_wait();
   fin_sync();
-  const T* emb_s = reinterpret_cast<const T*>(emb_raw);
-  for (int b = 0; b < st.B; ++b) {
-    if (threadIdx.x == 0 && (fs.tok_s[b] < 0 || fs.tok_s[b] >= st.vocab)) flag_status(st.status, DVI_DEV_BAD_TOKEN);
-    embed_row_block<T, NT>(emb_s + static_cast<size_t>(b) * st.d, 0, st.d, st.x_dr + static_cast<size_t>(b) * st.d,
-                       st.g0, static_cast<T*>(st.xg_dr) + static_cast<size_t>(b) * st.d, st.xg_dr_plane, st.ss_dr,
-                       st.ss_dr_ld, b, fs.red);
-  }
+  for (int b = threadIdx.x; b < st.B; b += kFinThreads)
+    if (fs.tok_s[b] < 0 || fs.tok_s[b] >= st.vocab) flag_status(st.status, DVI_DEV_BAD_TOKEN);
+  embed_rows<T>(st, fs.tok_s, reinterpret_cast<const T*>(emb_raw));
 }
 
 // Accept length, commit and rollback, the replay-buffer tuples' metadata,
@@ -271,7 +318,7 @@ __device__ void finalize_verify_body(const StepState& st, FinSmem& fs) {
       else flag_status(st.status, DVI_DEV_LOG_FULL);
     }
   }
-  embed_rows<T, NT>(st, fs.tok_s, fs.red);
+  embed_rows<T>(st, fs.tok_s);
 }
 
 // Greedy AR: the argmax is the next token of every sequence (finalize_ar).
@@ -286,7 +333,20 @@ __device__ void finalize_ar_body(const StepState& st, FinSmem& fs) {
     fs.tok_s[b] = y;
   }
   fin_sync();
-  embed_rows<T, NT>(st, fs.tok_s, fs.red);
+  embed_rows<T>(st, fs.tok_s);
+}
+
+// The drafter-head preparation of a draft pass whose finalize step runs in
+// the head: CTA b takes row b while the weights stream (only the finalize
+// step, after every CTA, overwrites the rows).  In the last CTA, row after
+// row, it and the embedding took 110 us of a 209 us head launch at batch 8.
+template <int NT>
+__device__ __forceinline__ void head_prepare(const FinArgs& f, float* red, float* rstd_s) {
+  if (f.kind != FIN_DRAFT || !f.prep) return;
+  for (int b = blockIdx.x; b < f.hp.rows; b += gridDim.x) {
+    prep_row<__nv_bfloat16, NT>(f.hp, b, true, red, rstd_s, nullptr);
+    fin_sync();
+  }
 }
 
 // The finalize step after a head projection, in the head's last CTA: every
@@ -305,7 +365,8 @@ __device__ __forceinline__ void head_finalize(const FinArgs& f, uint8_t* smem, i
   __threadfence();
   if (tid == 0) *f.ctr = 0;
   uint8_t* emb = f.stage ? smem + (sizeof(FinSmem) + 15) / 16 * 16 : nullptr;
-  if (f.kind == FIN_DRAFT) finalize_draft_body<__nv_bfloat16, NT>(f.st, f.j, f.hp, f.prep, fs, emb);
+  // (the preparation ran in the head's first CTAs)
+  if (f.kind == FIN_DRAFT) finalize_draft_body<__nv_bfloat16, NT>(f.st, f.j, f.hp, 0, fs, emb);
   else if (f.kind == FIN_VERIFY) finalize_verify_body<__nv_bfloat16, NT>(f.st, fs);
   else finalize_ar_body<__nv_bfloat16, NT>(f.st, fs);
 }

@@ -507,30 +507,87 @@ __global__ void __launch_bounds__(192, 2)
     compute_rstd(p, rstd, posn, tid, kTileRows);
     named_bar(1, kTileRows);
     if (p.lora_bmat) {
-      // B u of the LoRA term while the weights stream: warp w takes rows
-      // q = w, w + 4, ... of B; u = (x * rstd) * g, four features per lane
-      // per step, summed per lane in feature order then across the warp
-      for (int n = 0; n < p.M; ++n) {
-        const float r = rstd[n];
-        const float4* x4 = reinterpret_cast<const float4*>(p.bu_x + static_cast<size_t>(n) * p.bu_ldx);
+      // B u of the LoRA term while the weights stream: u = (x * rstd) * g, four
+      // features per lane per step, summed per lane in feature order then
+      // across the warp.  A finalizing head takes blocks: warp w rows 4 w ..
+      // 4 w + 3 of B (16 at most) against eight token rows at a time, so B and
+      // the rows are read once each.  (One (row, token) pair at a time took
+      // 165 us more than the weights at eight tokens of the 7B shape.)  The
+      // other instantiations, whose projections the blocks would cost 50 to 80
+      // registers, keep the pairs: heads split over K, of small vocabularies.
+      if constexpr (kFinNT > 0) {
+        constexpr int kBuTok = 8;
         const float4* g4 = reinterpret_cast<const float4*>(p.bu_g);
-        for (int q = warp; q < p.lora_r; q += 4) {
-          const float4* br = reinterpret_cast<const float4*>(p.lora_bmat + static_cast<size_t>(q) * p.K);
-          float acc = 0.f;
-#pragma unroll 4
-          for (int c = lane; c < p.K / 4; c += 32) {
-            const float4 b = br[c], xx = x4[c], gg = g4[c];
-            acc = fmaf(b.x, xx.x * r * gg.x, acc);
-            acc = fmaf(b.y, xx.y * r * gg.y, acc);
-            acc = fmaf(b.z, xx.z * r * gg.z, acc);
-            acc = fmaf(b.w, xx.w * r * gg.w, acc);
+        for (int t0 = 0; t0 < p.M; t0 += kBuTok) {
+          for (int q0 = 4 * warp; q0 < p.lora_r; q0 += kBuRank) {
+            float acc[kBuTok][4];
+#pragma unroll
+            for (int u = 0; u < kBuTok; ++u)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) acc[u][i] = 0.f;
+#pragma unroll 1
+            for (int c = lane; c < p.K / 4; c += 32) {
+              const float4 gg = g4[c];
+              float4 b[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i)   // (clamped, not skipped: all loads go out together)
+                b[i] = reinterpret_cast<const float4*>(p.lora_bmat +
+                                                       static_cast<size_t>(min(q0 + i, p.lora_r - 1)) * p.K)[c];
+              float4 x[kBuTok];
+#pragma unroll
+              for (int u = 0; u < kBuTok; ++u)
+                x[u] = reinterpret_cast<const float4*>(p.bu_x +
+                                                       static_cast<size_t>(min(t0 + u, p.M - 1)) * p.bu_ldx)[c];
+#pragma unroll
+              for (int u = 0; u < kBuTok; ++u) {
+                const float r = rstd[min(t0 + u, p.M - 1)];
+                const float4 y = make_float4(x[u].x * r * gg.x, x[u].y * r * gg.y, x[u].z * r * gg.z, x[u].w * r * gg.w);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  acc[u][i] = fmaf(b[i].x, y.x, acc[u][i]);
+                  acc[u][i] = fmaf(b[i].y, y.y, acc[u][i]);
+                  acc[u][i] = fmaf(b[i].z, y.z, acc[u][i]);
+                  acc[u][i] = fmaf(b[i].w, y.w, acc[u][i]);
+                }
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < kBuTok; ++u) {
+              if (t0 + u >= p.M) continue;
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const float t = warp_sum(acc[u][i]);
+                if (lane == 0 && q0 + i < p.lora_r) bu_s[(t0 + u) * p.lora_r + q0 + i] = t;
+              }
+            }
           }
-          acc = warp_sum(acc);
-          if (lane == 0) bu_s[n * p.lora_r + q] = acc;
+        }
+      } else {
+        for (int n = 0; n < p.M; ++n) {
+          const float r = rstd[n];
+          const float4* x4 = reinterpret_cast<const float4*>(p.bu_x + static_cast<size_t>(n) * p.bu_ldx);
+          const float4* g4 = reinterpret_cast<const float4*>(p.bu_g);
+          for (int q = warp; q < p.lora_r; q += 4) {
+            const float4* br = reinterpret_cast<const float4*>(p.lora_bmat + static_cast<size_t>(q) * p.K);
+            float acc = 0.f;
+#pragma unroll 4
+            for (int c = lane; c < p.K / 4; c += 32) {
+              const float4 b = br[c], xx = x4[c], gg = g4[c];
+              acc = fmaf(b.x, xx.x * r * gg.x, acc);
+              acc = fmaf(b.y, xx.y * r * gg.y, acc);
+              acc = fmaf(b.z, xx.z * r * gg.z, acc);
+              acc = fmaf(b.w, xx.w * r * gg.w, acc);
+            }
+            acc = warp_sum(acc);
+            if (lane == 0) bu_s[n * p.lora_r + q] = acc;
+          }
         }
       }
       named_bar(1, kTileRows);
     }
+    // (a head has no row positions: their place holds the partial sums)
+    if constexpr (kFinNT > 0)
+      head_prepare<kFinNT>(fin, reinterpret_cast<float*>(posn), reinterpret_cast<float*>(tmem_holder + 1));
     ok = mbar_wait(done, 0, p.status);
     tc_fence_after();
     const uint32_t lane_base = tmem + ((static_cast<uint32_t>(warp) * 32u) << 16);
@@ -565,7 +622,7 @@ __global__ void __launch_bounds__(192, 2)
     }
     // a head whose last CTA runs the pass's finalize step (the ring is free)
     if constexpr (!kSplit && kFinNT > 0) {
-      if (fin.kind != FIN_NONE) head_finalize<kFinNT>(fin, sA + abytes, tid);
+      if (fin.kind != FIN_NONE) head_finalize<kFinNT>(fin, sA, tid);
     }
   }
   if (kSplit) {
@@ -1264,7 +1321,7 @@ bool head_fin_ok(const ProjArgs& a, size_t stage_bytes, bool* stage) {
   size_t smem = 0;
   const int stages = tc_stages(a.n_pad, &smem);
   const size_t ring = static_cast<size_t>(stages) * (16384 + 2 * static_cast<size_t>(a.n_pad) * 128);
-  *stage = ring >= 16384 + fin_smem_bytes() + stage_bytes;
+  *stage = ring >= fin_smem_bytes() + stage_bytes;
   return ring >= 16384 + fin_smem_bytes();
 }
 

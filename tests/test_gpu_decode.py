@@ -20,7 +20,7 @@ import torch
 from oracle import OracleModel, greedy_ar, dvi_generate, DrafterUpdater
 from oracle.update import head_logits, grad_logits, param_grads, objective_weights, total_loss
 from workloads import workload, make_weights, make_prompts, tiny_shape, UpdateHyper
-from gpu_helpers import engine_for, rounded_weights, teacher_forced_logits
+from gpu_helpers import engine_for, logged_u, rounded_weights, teacher_forced_logits
 
 pytestmark = pytest.mark.gpu
 GOLD = json.load(open(os.path.join(os.path.dirname(__file__), "golden", "tiny_dvi.json")))
@@ -182,3 +182,31 @@ def test_prefill_chunks_do_not_change_results():
     ref = greedy_ar(m, P[0], w.gen_tokens)
     np.testing.assert_array_equal(outs[0], ref)
     np.testing.assert_array_equal(outs[1], ref)
+
+
+@pytest.mark.parametrize("batch,rank", [(3, 16), (9, 13), (16, 1)])
+def test_drafter_head_lora_blocks(batch, rank):
+    """B u formed by the finalizing head in blocks of eight tokens by four rows
+    of B: the logged z of one step against W^S u + gamma A (B u) in float64 from
+    the logged u.  z's products carry bf16 weights and hi + lo rows (2^-16 of
+    the row norm each way); 1e-4 of the largest z covers both."""
+    from paper_2510_05421_gb300 import DVIEngine, DeviceWeights
+    from workloads import tiny_shape
+    w = workload("tiny").with_(dtype="bf16", batch=batch, k_spec=2, lora_rank=rank, prompt_len=(5, 5), update_every=1,
+                               shape=tiny_shape(n_layers=2, vocab=20000), split_k=1)
+    W = make_weights(w)
+    g = np.random.default_rng(3)
+    W.lora_a[...] = g.standard_normal(W.lora_a.shape) * 0.05
+    eng = DVIEngine(w.shape, "bf16", DeviceWeights.from_host(W, "bf16"), batch=batch, k_spec=2, split_k=1,
+                    lora_rank=rank, max_seq_len=32, log_steps=1, use_graphs=False, megakernel=False)
+    for b, p in enumerate(make_prompts(w)):
+        eng.prefill(b, torch.from_numpy(p).cuda())
+    eng.step()
+    eng.sync()
+    u = logged_u(eng, w)
+    z = eng.buffer("Z", torch.float32).view(-1, w.shape.vocab).double().cpu().numpy()
+    assert eng.stats()["device_status"] == 0
+    eng.close()
+    ws = rounded_weights(W).draft_head.astype(np.float64)
+    ref = u @ ws.T + (u @ W.lora_b.astype(np.float64).T) @ W.lora_a.astype(np.float64).T
+    assert np.abs(z - ref).max() <= 1e-4 * np.abs(ref).max()
