@@ -32,7 +32,7 @@
 // fill the GPU.  bf16: the splits of a tile form one thread-block cluster;
 // each leaves its partial tile in shared memory and, after a cluster barrier,
 // rank r sums the partials of all ranks in rank order through distributed
-// shared memory for the token columns n = r (mod n_splits) and runs their
+// shared memory for its contiguous share of the token columns and runs their
 // epilogue.  f32: each split stores its partial in
 // global scratch and the last CTA to arrive (an atomic counter per tile) sums
 // them in split order.  Both are deterministic, and the split plan depends on
@@ -627,8 +627,8 @@ __global__ void __launch_bounds__(192, 2)
   }
   if (kSplit) {
     // ---------------- split-K across the cluster: rank r finishes the token
-    // columns n with n % S == r, summing every rank's partial in rank order
-    // (all of a column's loads from the peers are issued before the sum)
+    // columns [r M / S, (r + 1) M / S), summing every rank's partial in rank
+    // order (all of a column's loads from the peers are issued before the sum)
     cluster_arrive_release();
     cluster_wait_acquire();
     if (warp < 4) {
@@ -637,20 +637,18 @@ __global__ void __launch_bounds__(192, 2)
       const uint32_t mine = smem_u32(part) + static_cast<uint32_t>(tid) * 4u;
 #pragma unroll
       for (int r = 0; r < 8; ++r) peer[r] = r < S ? mapa_shared(mine, r) : 0u;
-      const int nchunks = (p.M + kChunk - 1) / kChunk;
-      for (int c = 0; c < nchunks; ++c) {
-        // columns n of [c0, c0 + 16) with n = split (mod S)
-        const int c0 = c * kChunk, c1 = min(p.M, c0 + kChunk);
-        uint32_t own = 0;
-        for (int n = c0 + (split - c0 % S + S) % S; n < c1; n += S) own |= 1u << (n - c0);
-        if (!own) continue;
+      // (a contiguous share: 40 rows over 8 ranks are 5 columns of one chunk
+      // each; dealt out round robin they lay in all three chunks, whose
+      // epilogues cost 8 us more per launch)
+      const int n_end = p.M * (split + 1) / S;
+      for (int c0 = p.M * split / S; c0 < n_end; c0 += kChunk) {
+        const int cols = min(kChunk, n_end - c0);
         // one compact loop over the owned columns: the sum of every rank's
         // partial (in rank order) replaces this rank's own partial, which
         // only this rank reads for the columns it owns
 #pragma unroll 1
-        for (int j = 0; j < kChunk; ++j) {
-          if (!((own >> j) & 1u)) continue;
-          const uint32_t off = static_cast<uint32_t>((c * kChunk + j) * kTileRows) * 4u;
+        for (int j = 0; j < cols; ++j) {
+          const uint32_t off = static_cast<uint32_t>((c0 + j) * kTileRows) * 4u;
           float t[8];
 #pragma unroll
           for (int r = 0; r < 8; ++r) t[r] = r < S ? ld_cluster_f32(peer[r] + off) : 0.f;
@@ -658,12 +656,12 @@ __global__ void __launch_bounds__(192, 2)
 #pragma unroll
           for (int r = 1; r < 8; ++r)
             if (r < S) acc += t[r];
-          part[(c * kChunk + j) * kTileRows + tid] = acc;
+          part[(c0 + j) * kTileRows + tid] = acc;
         }
         float v[kChunk];
 #pragma unroll
-        for (int j = 0; j < kChunk; ++j) v[j] = ((own >> j) & 1u) ? part[(c * kChunk + j) * kTileRows + tid] : 0.f;
-        epilogue_chunk<__nv_bfloat16>(p, tile, tid, c * kChunk, v, rstd, posn, es, own, bu_s);
+        for (int j = 0; j < kChunk; ++j) v[j] = j < cols ? part[(c0 + j) * kTileRows + tid] : 0.f;
+        epilogue_chunk<__nv_bfloat16>(p, tile, tid, c0, v, rstd, posn, es, (1u << cols) - 1u, bu_s);
       }
     }
     // every rank keeps its shared memory until all have read it
