@@ -174,12 +174,13 @@ def check_linear_noalloc_args(w, x, y) -> None:
         raise ValueError("linear_noalloc: w must be bf16 or float32")
     if x.dtype != torch.float32 or y.dtype != torch.float32:
         raise ValueError("linear_noalloc: x and y must be float32")
-    if len(w.shape) != 2 or len(x.shape) != 2 or len(y.shape) != 2:
+    ws, xs, ys = w.shape, x.shape, y.shape
+    if len(ws) != 2 or len(xs) != 2 or len(ys) != 2:
         raise ValueError("linear_noalloc: w, x and y must be 2-D")
-    n, k = w.shape
-    m = x.shape[0]
-    if x.shape[1] != k or tuple(y.shape) != (m, n):
-        raise ValueError(f"linear_noalloc: shapes w {tuple(w.shape)}, x {tuple(x.shape)}, y {tuple(y.shape)} "
+    n, k = ws
+    m = xs[0]
+    if xs[1] != k or ys[0] != m or ys[1] != n:
+        raise ValueError(f"linear_noalloc: shapes w {tuple(ws)}, x {tuple(xs)}, y {tuple(ys)} "
                          "do not match y[M, N] = x[M, K] w[N, K]^T")
     if not 1 <= m <= 256 or n < 1 or k < 1:
         raise ValueError("linear_noalloc: needs 1 <= M <= 256 rows and a non-empty weight")
@@ -199,11 +200,19 @@ def linear_noalloc(w: torch.Tensor, x: torch.Tensor, y: torch.Tensor, stream=Non
     the library's status code (0 on success).
     """
     check_linear_noalloc_args(w, x, y)
-    dtype = DVI_BF16 if w.dtype == torch.bfloat16 else DVI_F32
-    with torch.cuda.device(w.device):
-        s = stream if stream is not None else torch.cuda.current_stream(w.device)
-        return lib().dvi_linear_noalloc(dtype, _ptr(w), w.shape[0], w.shape[1], _ptr(x), x.shape[0], _ptr(y),
-                                        ctypes.c_void_p(s.cuda_stream))
+    dev = w.device.index
+    if dev != torch.cuda.current_device():
+        with torch.cuda.device(dev):
+            return _linear_noalloc(w, x, y, dev, stream)
+    return _linear_noalloc(w, x, y, dev, stream)
+
+
+def _linear_noalloc(w, x, y, dev: int, stream) -> int:
+    # the raw handle of torch's current stream, without a Stream object around it
+    s = torch._C._cuda_getCurrentRawStream(dev) if stream is None else stream.cuda_stream
+    m, k = x.shape
+    return lib().dvi_linear_noalloc(DVI_BF16 if w.dtype == torch.bfloat16 else DVI_F32, w.data_ptr(), w.shape[0], k,
+                                    x.data_ptr(), m, y.data_ptr(), s)
 
 
 class DVIEngine:
