@@ -1467,7 +1467,7 @@ dvi_status dvi_update_drafter(dvi_ctx* ctx, const dvi_update_config* u) {
   // row statistics; the last row's CTA forms the loss and the coefficients
   DVI_CUDA(launch_update_rowstats(a, s));
   if (full) {
-    DVI_CUDA(launch_update_full(a, s));
+    DVI_CUDA(launch_update_full(a, ctx->n_sms, s));
     DVI_CUDA(launch_update_finish(a, s));
     ctx->launches += (ctx->r > 0 ? 1 : 0) + 5;
   } else {

@@ -272,7 +272,7 @@ cudaError_t launch_update_prep(const UpdateArgs& a, cudaStream_t s);
 cudaError_t launch_update_rowstats(const UpdateArgs& a, cudaStream_t s);
 cudaError_t launch_update_grad_a(const UpdateArgs& a, cudaStream_t s);
 cudaError_t launch_update_grad_b(const UpdateArgs& a, cudaStream_t s);
-cudaError_t launch_update_full(const UpdateArgs& a, cudaStream_t s);
+cudaError_t launch_update_full(const UpdateArgs& a, int n_sms, cudaStream_t s);
 // LoRA mode: everything after the logits GEMM in one cooperative launch of
 // ------------------------------------------------------------ draft-phase megakernel
 // One persistent launch (one CTA per SM, every CTA resident) runs the

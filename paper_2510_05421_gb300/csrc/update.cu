@@ -995,6 +995,75 @@ constexpr int kGwRows = 16;    // W^S rows per CTA (accumulators per thread: kGw
 constexpr int kGwCols = 512;   // W^S columns per CTA: 128 threads x 4 consecutive columns
 constexpr int kGwStage = 16;   // buffer rows staged in shared memory per round
 
+// Four consecutive logged values (a column that is a multiple of 4; d is a
+// multiple of 128 and the planes start 256 bytes aligned).
+__device__ __forceinline__ float4 gw_ld4(const float* p, size_t) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 gw_ld4(const __nv_bfloat16* p, size_t plane) {
+  const uint2 h = *reinterpret_cast<const uint2*>(p), l = *reinterpret_cast<const uint2*>(p + plane);
+  return make_float4(bf16_lo(h.x) + bf16_lo(l.x), bf16_hi(h.x) + bf16_hi(l.x), bf16_lo(h.y) + bf16_lo(l.y),
+                     bf16_hi(h.y) + bf16_hi(l.y));
+}
+
+// W^S (its f32 master), m and v of four consecutive rows at columns c .. c + 3.
+struct GwRows4 {
+  float4 p[4], m[4], s[4];
+};
+__device__ __forceinline__ float* gw_master(const UpdateArgs& a) {
+  return a.w_master ? a.w_master : static_cast<float*>(a.w_head);
+}
+__device__ __forceinline__ void gw_load(const UpdateArgs& a, int v0, int c, GwRows4& r) {
+  const float* master = gw_master(a);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (v0 + j >= a.V) continue;
+    const size_t i = static_cast<size_t>(v0 + j) * a.d + c;
+    r.p[j] = *reinterpret_cast<const float4*>(master + i);
+    if (a.cfg.optimizer == 0) {
+      r.m[j] = *reinterpret_cast<const float4*>(a.m_w + i);
+      r.s[j] = *reinterpret_cast<const float4*>(a.v_w + i);
+    }
+  }
+}
+// The optimizer step on them with gradients g[0..3] (rows below `hi` only).
+__device__ __forceinline__ void gw_step(const UpdateArgs& a, int v0, int c, const GwRows4& r, const float4* grad,
+                                        int hi = 1 << 30) {
+  const dvi_update_config& cf = a.cfg;
+  const float bc1 = a.dev_state[DS_BC1], bc2 = a.dev_state[DS_BC2];
+  float* master = gw_master(a);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int v = v0 + j;
+    if (v >= a.V || v >= hi) continue;
+    const size_t i = static_cast<size_t>(v) * a.d + c;
+    const float4 g = grad[j];
+    if (a.keep_grad_w) *reinterpret_cast<float4*>(a.grad_w + i) = g;
+    float gv[4] = {g.x, g.y, g.z, g.w};
+    float pv[4] = {r.p[j].x, r.p[j].y, r.p[j].z, r.p[j].w};
+    if (cf.optimizer == 1) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) pv[q] -= cf.lr * gv[q];
+    } else {
+      float mv[4] = {r.m[j].x, r.m[j].y, r.m[j].z, r.m[j].w};
+      float sv[4] = {r.s[j].x, r.s[j].y, r.s[j].z, r.s[j].w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        mv[q] = cf.beta1 * mv[q] + (1.f - cf.beta1) * gv[q];
+        sv[q] = cf.beta2 * sv[q] + (1.f - cf.beta2) * gv[q] * gv[q];
+        pv[q] -= cf.lr * (mv[q] / bc1) / (sqrtf(sv[q] / bc2) + cf.adam_eps);
+      }
+      *reinterpret_cast<float4*>(a.m_w + i) = make_float4(mv[0], mv[1], mv[2], mv[3]);
+      *reinterpret_cast<float4*>(a.v_w + i) = make_float4(sv[0], sv[1], sv[2], sv[3]);
+    }
+    *reinterpret_cast<float4*>(master + i) = make_float4(pv[0], pv[1], pv[2], pv[3]);
+    if (a.w_master) {
+      uint2 packed;
+      packed.x = pack_bf16x2(pv[0], pv[1]);
+      packed.y = pack_bf16x2(pv[2], pv[3]);
+      *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(a.w_head) + i) = packed;
+    }
+  }
+}
+
 // dW = G^T U for a [kGwRows x kGwCols] tile of W^S, then the optimizer step
 // on it.  The contraction runs over the buffer rows (N <= 256), so it is a
 // few FMAs per W^S entry; the kernel streams W^S (master), m and v once.
@@ -1048,55 +1117,70 @@ __global__ void __launch_bounds__(128) update_gw_kernel(const UpdateArgs a) {
     }
   }
   if (c >= a.d) return;
-  const dvi_update_config& cf = a.cfg;
-  const float bc1 = a.dev_state[DS_BC1], bc2 = a.dev_state[DS_BC2];
-  float* master = a.w_master ? a.w_master : static_cast<float*>(a.w_head);
   // four rows at a time: their loads are issued before any store
 #pragma unroll
   for (int g0 = 0; g0 < kGwRows; g0 += 4) {
-    float4 p[4], m[4], s[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int v = v0 + g0 + j;
-      if (v >= a.V) continue;
-      const size_t i = static_cast<size_t>(v) * a.d + c;
-      p[j] = *reinterpret_cast<const float4*>(master + i);
-      if (cf.optimizer == 0) {
-        m[j] = *reinterpret_cast<const float4*>(a.m_w + i);
-        s[j] = *reinterpret_cast<const float4*>(a.v_w + i);
-      }
+    GwRows4 r;
+    gw_load(a, v0 + g0, c, r);
+    gw_step(a, v0 + g0, c, r, &acc[g0]);
+  }
+}
+
+// The same for a buffer of few rows: a CTA keeps its 512 columns of U in
+// shared memory and walks a long run of W^S rows, four at a time, with the
+// next four rows' W^S, m and v in flight during the contraction and the step.
+// Bound by HBM: 26 B per entry of a bf16 W^S (1.70 GB at 32000 x 2048, 20
+// buffer rows): 334 us, 5.1 TB/s; the kernel above, which stages U again for
+// every 16 rows and has nothing in flight meanwhile, 468 us.
+// grid = (row runs, ceil(d / kGwCols)), 128 threads.
+constexpr int kGwResRows = 32;    // largest buffer whose U is kept (64 KB of 512 columns)
+constexpr int kGwResBlock = 64;   // W^S rows whose logit gradients are staged together
+template <typename T>
+__global__ void __launch_bounds__(128) update_gw_res_kernel(const UpdateArgs a, int rows_per_cta) {
+  extern __shared__ __align__(16) float gw_smem[];
+  griddep_launch();
+  griddep_wait();
+  if (a.dev_state[DS_SKIP] != 0.f) return;
+  float4* us = reinterpret_cast<float4*>(gw_smem);                  // [cap][128]
+  float* gs = gw_smem + static_cast<size_t>(a.cap) * kGwCols;      // [cap][kGwResBlock]
+  const int tid = threadIdx.x;
+  const int c = blockIdx.y * kGwCols + tid * 4;
+  const int lo = blockIdx.x * rows_per_cta, hi = min(a.V, lo + rows_per_cta);
+  const T* U = static_cast<const T*>(a.log_u);
+  const bool on = c < a.d;
+  for (int n = 0; n < a.cap; ++n)
+    us[n * 128 + tid] = on && row_valid(a, n) ? gw_ld4(U + static_cast<size_t>(n) * a.d + c, a.log_plane)
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+  GwRows4 r;
+  if (on) gw_load(a, lo, c, r);
+  for (int b0 = lo; b0 < hi; b0 += kGwResBlock) {
+    __syncthreads();   // the block before is done with gs
+    for (int i = tid; i < a.cap * kGwResBlock; i += 128) {
+      const int n = i / kGwResBlock, v = b0 + i % kGwResBlock;
+      gs[i] = v < hi ? a.G[static_cast<size_t>(n) * a.V + v] : 0.f;
     }
+    __syncthreads();
+    if (!on) continue;
+    for (int v0 = b0; v0 < min(hi, b0 + kGwResBlock); v0 += 4) {
+      const GwRows4 cur = r;
+      if (v0 + 4 < hi) gw_load(a, v0 + 4, c, r);
+      float4 acc[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int v = v0 + g0 + j;
-      if (v >= a.V) continue;
-      const size_t i = static_cast<size_t>(v) * a.d + c;
-      const float4 g = acc[g0 + j];
-      if (a.keep_grad_w) *reinterpret_cast<float4*>(a.grad_w + i) = g;
-      float gv[4] = {g.x, g.y, g.z, g.w};
-      float pv[4] = {p[j].x, p[j].y, p[j].z, p[j].w};
-      if (cf.optimizer == 1) {
+      for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+      for (int n = 0; n < a.cap; ++n) {
+        const float4 u = us[n * 128 + tid];
+        const float4 g4 = *reinterpret_cast<const float4*>(gs + n * kGwResBlock + (v0 - b0));
+        const float g[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) pv[q] -= cf.lr * gv[q];
-      } else {
-        float mv[4] = {m[j].x, m[j].y, m[j].z, m[j].w};
-        float sv[4] = {s[j].x, s[j].y, s[j].z, s[j].w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          mv[q] = cf.beta1 * mv[q] + (1.f - cf.beta1) * gv[q];
-          sv[q] = cf.beta2 * sv[q] + (1.f - cf.beta2) * gv[q] * gv[q];
-          pv[q] -= cf.lr * (mv[q] / bc1) / (sqrtf(sv[q] / bc2) + cf.adam_eps);
+        for (int i = 0; i < 4; ++i) {
+          acc[i].x = fmaf(g[i], u.x, acc[i].x);
+          acc[i].y = fmaf(g[i], u.y, acc[i].y);
+          acc[i].z = fmaf(g[i], u.z, acc[i].z);
+          acc[i].w = fmaf(g[i], u.w, acc[i].w);
         }
-        *reinterpret_cast<float4*>(a.m_w + i) = make_float4(mv[0], mv[1], mv[2], mv[3]);
-        *reinterpret_cast<float4*>(a.v_w + i) = make_float4(sv[0], sv[1], sv[2], sv[3]);
       }
-      *reinterpret_cast<float4*>(master + i) = make_float4(pv[0], pv[1], pv[2], pv[3]);
-      if (a.w_master) {
-        uint2 packed;
-        packed.x = pack_bf16x2(pv[0], pv[1]);
-        packed.y = pack_bf16x2(pv[2], pv[3]);
-        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(a.w_head) + i) = packed;
-      }
+      gw_step(a, v0, c, cur, acc, hi);
     }
   }
 }
@@ -1182,10 +1266,27 @@ cudaError_t launch_update_fused(const UpdateArgs& a, int n_sms, cudaStream_t s) 
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_update_full(const UpdateArgs& a, cudaStream_t s) {
+cudaError_t launch_update_full(const UpdateArgs& a, int n_sms, cudaStream_t s) {
   cudaError_t e = launch_pdl(update_g_kernel, dim3((a.V + 255) / 256, a.cap), dim3(256), 0, s, a);
   if (e != cudaSuccess) return e;
-  const dim3 grid((a.V + kGwRows - 1) / kGwRows, (a.d + kGwCols - 1) / kGwCols);
+  const int cblocks = (a.d + kGwCols - 1) / kGwCols;
+  if (a.cap <= kGwResRows) {
+    // three CTAs per SM (registers); runs of whole row quads
+    const int runs = std::max(1, 3 * n_sms / cblocks);
+    const int per = std::max(4, ((a.V + runs - 1) / runs + 3) / 4 * 4);
+    const dim3 rgrid((a.V + per - 1) / per, cblocks);
+    const size_t smem = sizeof(float) * static_cast<size_t>(a.cap) * (kGwCols + kGwResBlock);
+    static PerDevice attr;
+    attr.once([] {
+      const int most = static_cast<int>(sizeof(float)) * kGwResRows * (kGwCols + kGwResBlock);
+      cudaFuncSetAttribute(update_gw_res_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+      cudaFuncSetAttribute(update_gw_res_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    });
+    e = a.dtype == DVI_BF16 ? launch_pdl(update_gw_res_kernel<__nv_bfloat16>, rgrid, dim3(128), smem, s, a, per)
+                            : launch_pdl(update_gw_res_kernel<float>, rgrid, dim3(128), smem, s, a, per);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
+  const dim3 grid((a.V + kGwRows - 1) / kGwRows, cblocks);
   e = a.dtype == DVI_BF16 ? launch_pdl(update_gw_kernel<__nv_bfloat16>, grid, dim3(128), 0, s, a)
                           : launch_pdl(update_gw_kernel<float>, grid, dim3(128), 0, s, a);
   if (e != cudaSuccess) return e;

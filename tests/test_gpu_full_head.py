@@ -11,6 +11,8 @@ of Sec. 3.4.  Checked against the oracle:
   dL/dW^(S) of one update against the oracle on the GPU's own logged tuples,
   and the bf16 head equals the rounding of the f32 master.
 """
+from dataclasses import replace
+
 import numpy as np
 import pytest
 import torch
@@ -121,3 +123,29 @@ def test_bf16_full_head_lossless_and_gradient():
     step = np.abs(w_new - w_s)
     assert np.median(step) > 0.25 * hyper.lr and step.max() < 4 * hyper.lr
     assert torch.equal(torch.from_numpy(w_new).bfloat16().float(), torch.from_numpy(w_new))
+
+
+@pytest.mark.parametrize("steps,vocab", [(7, 1021), (8, 1024), (12, 1021)])
+def test_gradient_tiles(steps, vocab):
+    """dL/dW^(S) and the step by both kernels: U kept in shared memory (buffers
+    of 28 and 32 rows) and staged per tile (48 rows), a vocabulary that ends
+    inside a row quad and a d that ends inside a column block (640 = 512 + 128)."""
+    w = workload("tiny").with_(update_every=steps)
+    w = w.with_(shape=replace(w.shape, d_model=640, vocab=vocab))
+    hyper = UpdateHyper(objective="kl", lr=1e-3)
+    W = make_weights(w)
+    P = make_prompts(w)
+    eng, _, dw = engine_for(w, W=W, head_mode=1)
+    w_before = dw.draft_head.cpu().numpy().copy()
+    eng.generate(P, 10 ** 6, max_steps=steps, log=True)
+    eng.update(hyper, keep_grad_w=True)
+    eng.sync()
+    gw = eng.buffer("GRAD_W", torch.float32).view(vocab, -1).cpu().numpy()
+    w_after = dw.draft_head.cpu().numpy().copy()
+    assert eng.stats()["device_status"] == 0
+    eng.close()
+    m = OracleModel(W, w.shape, w.lora_gamma)
+    res = dvi_generate(m, P, 10 ** 6, w.split_k, w.k_spec, steps, Recorder(m, hyper, full=True), max_steps=steps)
+    g_ref = res.updates[0]["grads"]["W_s"]
+    assert np.abs(gw - g_ref).max() <= 1e-3 * np.abs(g_ref).max()
+    _check_step(w_after, w_before, g_ref, hyper.lr)
