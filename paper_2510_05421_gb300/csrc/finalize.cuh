@@ -32,6 +32,9 @@ __device__ __forceinline__ void fin_sync() { named_bar(2, kFinThreads); }
 // Shared memory of a finalize step.
 struct FinSmem {
   int tok_s[64];
+  int m_s[64];                    // verify: accept lengths,
+  int y_s[kMaxTokens];            // y* of every verify row,
+  int dr_s[kMaxTokens + 64];      // and the block's tokens [B][K + 1]
   float red[kMaxTiles * 4];
   float rstd_s;
   int last;   // head projection: this CTA is the last to finish
@@ -274,42 +277,47 @@ __device__ void finalize_draft_body(const StepState& st, int j, const HeadPrepAr
 template <typename T, int NT = kMaxTiles>
 __device__ void finalize_verify_body(const StepState& st, FinSmem& fs) {
   const int K = st.K, Kv = st.Kv;
+  // one round trip: every row's argmax and every drafted token by a thread of
+  // its own (a sequence's thread reading them in turn took 10 us)
+  for (int t = threadIdx.x; t < st.B * Kv; t += kFinThreads) fs.y_s[t] = take_argmax(st.amax + t, st.status);
+  for (int t = threadIdx.x; t < st.B * (K + 1); t += kFinThreads) fs.dr_s[t] = st.draft_ids[t];
   const int ls = *st.log_step;
   const bool log_ok = st.log_enabled && ls < st.log_cap_steps;
+  fin_sync();
   for (int b = threadIdx.x; b < st.B; b += kFinThreads) {
-    int y[16];
-    for (int i = 0; i < Kv; ++i) y[i] = take_argmax(st.amax + b * Kv + i, st.status);
-    int* dr = st.draft_ids + b * (K + 1);
+    const int* y = fs.y_s + b * Kv;
+    const int* dr = fs.dr_s + b * (K + 1);
     int m = 0;
     while (m < K && dr[m + 1] == y[m]) ++m;
     // the correction y*_{n+m+1} exists for m < K, and for m = K with the bonus row
     const int c = m < Kv ? m + 1 : K;
-    for (int i = 0; i < Kv; ++i) {
-      const int id = i < m ? dr[i + 1] : (i == m ? y[m] : -1);
-      st.out_ids[b * Kv + i] = id;
-    }
+    const int newtok = m < Kv ? y[m] : dr[K];
     st.n_committed[b] = c;
     st.n_accepted[b] = m;
-    if (log_ok) {
-      for (int i = 0; i < K; ++i) {
-        int* meta = st.log_meta + (static_cast<size_t>(ls) * st.B * K + b * K + i) * 6;
-        meta[0] = i < c;
-        meta[1] = dr[i + 1];
-        meta[2] = i < m ? 1 : 0;
-        meta[3] = i + 1;
-        meta[4] = dr[i];
-        meta[5] = y[i];
-      }
-    }
-    const int newtok = st.out_ids[b * Kv + c - 1];
     st.lens[b] += c;
     st.pending[b] = newtok;
-    dr[0] = newtok;
+    st.draft_ids[b * (K + 1)] = newtok;
     fs.tok_s[b] = newtok;
+    fs.m_s[b] = m;
     atomicAdd(reinterpret_cast<unsigned long long*>(st.counters + 2), static_cast<unsigned long long>(m));
     atomicAdd(reinterpret_cast<unsigned long long*>(st.counters + 3), static_cast<unsigned long long>(c));
   }
   fin_sync();
+  for (int t = threadIdx.x; t < st.B * Kv; t += kFinThreads) {
+    const int b = t / Kv, i = t % Kv, m = fs.m_s[b];
+    const int* dr = fs.dr_s + b * (K + 1);
+    st.out_ids[t] = i < m ? dr[i + 1] : (i == m ? fs.y_s[t] : -1);
+    if (log_ok && i < K) {
+      const int c = m < Kv ? m + 1 : K;
+      int* meta = st.log_meta + (static_cast<size_t>(ls) * st.B * K + b * K + i) * 6;
+      meta[0] = i < c;
+      meta[1] = dr[i + 1];
+      meta[2] = i < m ? 1 : 0;
+      meta[3] = i + 1;
+      meta[4] = dr[i];
+      meta[5] = fs.y_s[t];
+    }
+  }
   if (threadIdx.x == 0) {
     st.counters[0] += 1;
     st.counters[1] += static_cast<long long>(st.B) * K;

@@ -102,12 +102,38 @@ __device__ __forceinline__ uint32_t valid_cols(const ProjArgs& p, int c0) {
   return n >= kChunk ? 0xffffu : ((1u << max(n, 0)) - 1u);
 }
 
+// What an epilogue reads per owned column besides the accumulators, all loads
+// in flight together and, where the caller can, ahead of the accumulator: the
+// rotation (cos, sin) of the thread's dim at the column's position (QKV), the
+// residual (RESID, in .x).  Read column by column inside the epilogue they
+// were a round trip each.
+template <typename T>
+__device__ __forceinline__ void epi_pre(const ProjArgs& p, int tile, int row, int c0, uint32_t own, const int* posn,
+                                        float2 (&pre)[kChunk]) {
+  if (p.flavor == EPI_QKV) {
+    const int half = p.head_dim >> 1;
+    const bool rot = tile < (p.rows_q + p.rows_k) / kTileRows;
+    const float2* rope = p.rope + (tile * kTileRows + row) % half;   // sections are multiples of the head dim
+#pragma unroll
+    for (int j = 0; j < kChunk; ++j) {
+      const int pos = (own >> j) & 1u ? posn[c0 + j] : 0;
+      pre[j] = rot && pos >= 0 && pos < p.max_len ? rope[static_cast<size_t>(pos) * half] : make_float2(1.f, 0.f);
+    }
+  } else if (p.flavor == EPI_RESID) {
+    const int f = tile * kTileRows + row;
+    const float* x = p.x_res + static_cast<size_t>(c0) * p.ld_res + f;
+#pragma unroll
+    for (int j = 0; j < kChunk; ++j)
+      pre[j].x = ((own >> j) & 1u) && f < p.n_out ? __ldcg(x + static_cast<size_t>(j) * p.ld_res) : 0.f;
+  }
+}
+
 // Fused epilogue for the token columns of [c0, c0+16) set in `own` (a
 // subset of the valid ones) of one 128-feature tile.  Called by the 128
 // epilogue threads together (row = feature within tile).
 template <typename T>
 __device__ __forceinline__ void epilogue_chunk(const ProjArgs& p, int tile, int row, int c0, float (&v)[kChunk],
-                               const float* rstd, const int* posn, EpiSmem& es, uint32_t own,
+                               const float2 (&pre)[kChunk], const float* rstd, const int* posn, EpiSmem& es, uint32_t own,
                                const float* bu_s = nullptr) {
   const int warp = row >> 5, lane = row & 31;
   if (p.ss) {
@@ -143,7 +169,7 @@ __device__ __forceinline__ void epilogue_chunk(const ProjArgs& p, int tile, int 
           float val = v[j];
           if (sec < 2) {
             const float vp = es.stage[prow][j];
-            const float2 cs = p.rope[static_cast<size_t>(pos) * half + (dim % half)];
+            const float2 cs = pre[j];
             val = dim < half ? val * cs.x - vp * cs.y : val * cs.x + vp * cs.y;
           }
           if (sec == 0) {
@@ -165,9 +191,8 @@ __device__ __forceinline__ void epilogue_chunk(const ProjArgs& p, int tile, int 
       const int n = c0 + j;
       float xn = 0.f;
       if (((own >> j) & 1u) && f < p.n_out) {
-        float* xp = p.x_res + static_cast<size_t>(n) * p.ld_res + f;
-        xn = __ldcg(xp) + v[j];
-        *xp = xn;
+        xn = pre[j].x + v[j];
+        p.x_res[static_cast<size_t>(n) * p.ld_res + f] = xn;
         if (p.xg_out) Act<T>::st(static_cast<T*>(p.xg_out) + static_cast<size_t>(n) * p.ld_xg + f, p.xg_plane, xn * g);
       }
       sq[j] = xn * xn;
@@ -187,14 +212,16 @@ __device__ __forceinline__ void epilogue_chunk(const ProjArgs& p, int tile, int 
 #pragma unroll
     for (int j = 0; j < kChunk; ++j) es.stage[row][j] = v[j];
     named_bar(1, kTileRows);
-    const int f = tile * kGuRows + row;
-    if (row < kGuRows && f < p.n_out) {
+    // threads r and r + 64 take the feature's columns 0..7 and 8..15
+    const int fr = row & (kGuRows - 1), j0 = row >= kGuRows ? kChunk / 2 : 0;
+    const int f = tile * kGuRows + fr;
+    if (f < p.n_out) {
 #pragma unroll
-      for (int j = 0; j < kChunk; ++j) {
-        const int n = c0 + j;
+      for (int e = 0; e < kChunk / 2; ++e) {
+        const int j = j0 + e, n = c0 + j;
         if ((own >> j) & 1u) {
-          const float gt = es.stage[row][j];
-          const float h = gt / (1.f + expf(-gt)) * es.stage[row + kGuRows][j];
+          const float gt = es.stage[fr][j];
+          const float h = gt / (1.f + expf(-gt)) * es.stage[fr + kGuRows][j];
           Act<T>::st(static_cast<T*>(p.h_out) + static_cast<size_t>(n) * p.ld_h + f, p.h_plane, h);
         }
       }
@@ -396,6 +423,10 @@ __global__ void __launch_bounds__(192, 2)
   griddep_launch();
   const uint32_t tmem = *tmem_holder;
   bool ok = true;
+  // token columns this split finishes, and their first chunk's operands
+  const int n_lo = p.M * split / S, n_end = p.M * (split + 1) / S;
+  const uint32_t first_own = n_end - n_lo >= kChunk ? 0xffffu : (1u << (n_end - n_lo)) - 1u;
+  float2 pre[kChunk];
 
   if (warp == 4) {
     // ---------------- TMA producer: weight tile (+ activation tile) per stage
@@ -588,6 +619,8 @@ __global__ void __launch_bounds__(192, 2)
     // (a head has no row positions: their place holds the partial sums)
     if constexpr (kFinNT > 0)
       head_prepare<kFinNT>(fin, reinterpret_cast<float*>(posn), reinterpret_cast<float*>(tmem_holder + 1));
+    // a split's first columns: their operands arrive while the weights stream
+    if (kSplit) epi_pre<__nv_bfloat16>(p, tile, tid, n_lo, first_own, posn, pre);
     ok = mbar_wait(done, 0, p.status);
     tc_fence_after();
     const uint32_t lane_base = tmem + ((static_cast<uint32_t>(warp) * 32u) << 16);
@@ -600,9 +633,12 @@ __global__ void __launch_bounds__(192, 2)
         tmem_ld16(lane_base + p.n_pad + c * kChunk, vl);
 #pragma unroll
         for (int j = 0; j < kChunk; ++j) v[j] += vl[j];
-        if (ok)
-          epilogue_chunk<__nv_bfloat16>(p, tile, tid, c * kChunk, v, rstd, posn, es, valid_cols(p, c * kChunk),
-                                        bu_s);
+        if (ok) {
+          float2 pre[kChunk];
+          epi_pre<__nv_bfloat16>(p, tile, tid, c * kChunk, valid_cols(p, c * kChunk), posn, pre);
+          epilogue_chunk<__nv_bfloat16>(p, tile, tid, c * kChunk, v, pre, rstd, posn, es,
+                                        valid_cols(p, c * kChunk), bu_s);
+        }
       }
     } else {
       for (int c = 0; c < nchunks; ++c) {
@@ -640,9 +676,9 @@ __global__ void __launch_bounds__(192, 2)
       // (a contiguous share: 40 rows over 8 ranks are 5 columns of one chunk
       // each; dealt out round robin they lay in all three chunks, whose
       // epilogues cost 8 us more per launch)
-      const int n_end = p.M * (split + 1) / S;
-      for (int c0 = p.M * split / S; c0 < n_end; c0 += kChunk) {
+      for (int c0 = n_lo; c0 < n_end; c0 += kChunk) {
         const int cols = min(kChunk, n_end - c0);
+        if (c0 > n_lo) epi_pre<__nv_bfloat16>(p, tile, tid, c0, (1u << cols) - 1u, posn, pre);
         // one compact loop over the owned columns: the sum of every rank's
         // partial (in rank order) replaces this rank's own partial, which
         // only this rank reads for the columns it owns
@@ -661,7 +697,7 @@ __global__ void __launch_bounds__(192, 2)
         float v[kChunk];
 #pragma unroll
         for (int j = 0; j < kChunk; ++j) v[j] = j < cols ? part[(c0 + j) * kTileRows + tid] : 0.f;
-        epilogue_chunk<__nv_bfloat16>(p, tile, tid, c0, v, rstd, posn, es, (1u << cols) - 1u, bu_s);
+        epilogue_chunk<__nv_bfloat16>(p, tile, tid, c0, v, pre, rstd, posn, es, (1u << cols) - 1u, bu_s);
       }
     }
     // every rank keeps its shared memory until all have read it
@@ -988,7 +1024,10 @@ __global__ void __launch_bounds__(192, 2) proj_chain_kernel(const __grid_constan
             tmem_ld16(lane_base + n_pad + c * kChunk, vl);
 #pragma unroll
             for (int j = 0; j < kChunk; ++j) v[j] += vl[j];
-            epilogue_chunk<__nv_bfloat16>(p, tile, tid, c * kChunk, v, rstd, posn, es, valid_cols(p, c * kChunk));
+            float2 pre[kChunk];
+            epi_pre<__nv_bfloat16>(p, tile, tid, c * kChunk, valid_cols(p, c * kChunk), posn, pre);
+            epilogue_chunk<__nv_bfloat16>(p, tile, tid, c * kChunk, v, pre, rstd, posn, es,
+                                          valid_cols(p, c * kChunk));
           }
           tc_fence_before();
           named_bar(1, kTileRows);
@@ -1065,7 +1104,9 @@ __global__ void __launch_bounds__(192, 2) proj_chain_kernel(const __grid_constan
               }
 #pragma unroll
               for (int j = 0; j < kChunk; ++j) v[j] = ((own >> j) & 1u) ? v[j] : 0.f;
-              epilogue_chunk<__nv_bfloat16>(p, tile, tid, c * kChunk, v, rstd, posn, es, own);
+              float2 pre[kChunk];
+              epi_pre<__nv_bfloat16>(p, tile, tid, c * kChunk, own, posn, pre);
+              epilogue_chunk<__nv_bfloat16>(p, tile, tid, c * kChunk, v, pre, rstd, posn, es, own);
             }
             tc_fence_before();
             named_bar(1, kTileRows);
@@ -1228,8 +1269,10 @@ __global__ void __launch_bounds__(128) proj_f32_kernel(const ProjArgs p) {
   // rstd[c0 + j] is this tile's
   float* rs = rstd - c0;
   const int* ps = posn - c0;
+  float2 pre[kChunk];
+  epi_pre<float>(p, tile, row, c0, valid_cols(p, c0), ps, pre);
   if (p.n_splits == 1) {
-    epilogue_chunk<float>(p, tile, row, c0, acc, rs, ps, es, valid_cols(p, c0));
+    epilogue_chunk<float>(p, tile, row, c0, acc, pre, rs, ps, es, valid_cols(p, c0));
     return;
   }
   const size_t reg = static_cast<size_t>(kTileRows) * kChunk;
@@ -1255,7 +1298,7 @@ __global__ void __launch_bounds__(128) proj_f32_kernel(const ProjArgs p) {
       for (int j = 0; j < NJ; ++j)
         if (s0 + u < p.n_splits) acc[j] += t[u][j];
   }
-  epilogue_chunk<float>(p, tile, row, c0, acc, rs, ps, es, valid_cols(p, c0));
+  epilogue_chunk<float>(p, tile, row, c0, acc, pre, rs, ps, es, valid_cols(p, c0));
 }
 
 // ------------------------------------------------------------------ host
