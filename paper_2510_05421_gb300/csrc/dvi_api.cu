@@ -1370,12 +1370,10 @@ dvi_status dvi_draft_verify_commit(dvi_ctx* ctx, int32_t* d_out_ids, int32_t* d_
   rc = run_graph(ctx, &ctx->verify_exec, &ctx->verify_launches, g, [&] { return enqueue_verify(ctx); });
   if (rc != DVI_OK) return rc;
   mark_end(ctx, 1, t1);
-  if (d_out_ids)
-    DVI_CUDA(cudaMemcpyAsync(d_out_ids, ctx->out_ids, sizeof(int) * ctx->B * ctx->Kv, cudaMemcpyDeviceToDevice, s));
-  if (d_n_committed)
-    DVI_CUDA(cudaMemcpyAsync(d_n_committed, ctx->n_committed, sizeof(int) * ctx->B, cudaMemcpyDeviceToDevice, s));
-  if (d_n_accepted)
-    DVI_CUDA(cudaMemcpyAsync(d_n_accepted, ctx->n_accepted, sizeof(int) * ctx->B, cudaMemcpyDeviceToDevice, s));
+  if (d_out_ids || d_n_committed || d_n_accepted) {
+    DVI_CUDA(launch_copy_out(step_state(ctx), d_out_ids, d_n_committed, d_n_accepted, s));
+    ctx->launches += 1;
+  }
   return DVI_OK;
 }
 

@@ -158,17 +158,13 @@ __device__ __forceinline__ int take_argmax(unsigned long long* slot, int* status
 
 // Four consecutive values (a column that is a multiple of 4); one vector load
 // where the row's address allows it.
-__device__ __forceinline__ float4 ld_row4(const float* p, bool vec) {
-  return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
-}
 __device__ __forceinline__ float4 ld_row4(const __nv_bfloat16* p, bool vec) {
   if (!vec) return make_float4(__bfloat162float(p[0]), __bfloat162float(p[1]), __bfloat162float(p[2]),
                                __bfloat162float(p[3]));
   const uint2 u = *reinterpret_cast<const uint2*>(p);
   return make_float4(bf16_lo(u.x), bf16_hi(u.x), bf16_lo(u.y), bf16_hi(u.y));
 }
-// The activation row's four values at p (hi and lo planes for bf16).
-__device__ __forceinline__ void st_act_row4(float* p, size_t, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+// The activation row's four values at p (hi and lo planes).
 __device__ __forceinline__ void st_act_row4(__nv_bfloat16* p, size_t plane, float4 v) {
   uint2 hi, lo;
   split_bf16x2(v.x, v.y, hi.x, lo.x);
@@ -180,38 +176,59 @@ __device__ __forceinline__ void st_act_row4(__nv_bfloat16* p, size_t plane, floa
 // Embeds each sequence's next input token into the draft residual stream: x,
 // x * g and the per-tile sums of squares.  A warp per eight 128-feature tiles
 // of a row, four features of each a lane, its loads in flight together;
-// `staged`: the rows in shared memory, else they come from the table.  (One row after
+// `staged`: the rows in shared memory, else they come from the table.  f32
+// rows keep the order of their sums (a warp's 32 features at a time).  (One row after
 // another by all 128 threads took 14 us a row: 110 of a draft head's 162 us
 // at batch 8.)
 template <typename T>
 __device__ void embed_rows(const StepState& st, const int* toks, const T* staged = nullptr) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d = st.d, nt = d / kTileRows;
-  const bool gvec = (reinterpret_cast<uintptr_t>(st.g0) & 15u) == 0;
-  const bool svec = staged || (reinterpret_cast<uintptr_t>(st.embed) & 15u) == 0;
+  [[maybe_unused]] const bool svec = staged || (reinterpret_cast<uintptr_t>(st.embed) & 15u) == 0;
   const int parts = (nt + 7) / 8;
   for (int it = warp; it < st.B * parts; it += kFinThreads / 32) {
     const int b = it / parts, t0 = it % parts * 8;
     const T* src = (staged ? staged + static_cast<size_t>(b) * d
-                           : static_cast<const T*>(st.embed) + static_cast<size_t>(toks[b]) * d) + 4 * lane;
-    float* x = st.x_dr + static_cast<size_t>(b) * d + 4 * lane;
-    T* xg = static_cast<T*>(st.xg_dr) + static_cast<size_t>(b) * d + 4 * lane;
-    float4 v[8], g[8];
+                           : static_cast<const T*>(st.embed) + static_cast<size_t>(toks[b]) * d);
+    float* x = st.x_dr + static_cast<size_t>(b) * d;
+    T* xg = static_cast<T*>(st.xg_dr) + static_cast<size_t>(b) * d;
+    if constexpr (sizeof(T) == 4) {
+      for (int t = t0; t < min(t0 + 8, nt); ++t) {
+        float q[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int t = min(t0 + u, nt - 1);
-      v[u] = ld_row4(src + t * kTileRows, svec);
-      g[u] = ld_row4(st.g0 + t * kTileRows + 4 * lane, gvec);
-    }
+        for (int e = 0; e < 4; ++e) {
+          const int c = t * kTileRows + 32 * e + lane;
+          const float f = src[c];
+          x[c] = f;
+          xg[c] = f * st.g0[c];
+          q[e] = f * f;
+        }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int t = t0 + u;
-      if (t >= nt) break;
-      *reinterpret_cast<float4*>(x + t * kTileRows) = v[u];
-      st_act_row4(xg + t * kTileRows, st.xg_dr_plane,
-                  make_float4(v[u].x * g[u].x, v[u].y * g[u].y, v[u].z * g[u].z, v[u].w * g[u].w));
-      const float q = warp_sum((v[u].x * v[u].x + v[u].y * v[u].y) + (v[u].z * v[u].z + v[u].w * v[u].w));
-      if (lane == 0) st.ss_dr[static_cast<size_t>(t) * st.ss_dr_ld + b] = q;
+        for (int e = 0; e < 4; ++e) q[e] = warp_sum(q[e]);
+        if (lane == 0) st.ss_dr[static_cast<size_t>(t) * st.ss_dr_ld + b] = (q[0] + q[1]) + (q[2] + q[3]);
+      }
+    } else {
+      src += 4 * lane;
+      x += 4 * lane;
+      xg += 4 * lane;
+      float4 v[8], g[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = min(t0 + u, nt - 1);
+        v[u] = ld_row4(src + t * kTileRows, svec);
+        const float* gp = st.g0 + t * kTileRows + 4 * lane;   // 16-byte aligned (bf16 models)
+        g[u] = *reinterpret_cast<const float4*>(gp);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = t0 + u;
+        if (t >= nt) break;
+        *reinterpret_cast<float4*>(x + t * kTileRows) = v[u];
+        st_act_row4(xg + t * kTileRows, st.xg_dr_plane,
+                    make_float4(v[u].x * g[u].x, v[u].y * g[u].y, v[u].z * g[u].z, v[u].w * g[u].w));
+        const float q = warp_sum((v[u].x * v[u].x + v[u].y * v[u].y) + (v[u].z * v[u].z + v[u].w * v[u].w));
+        if (lane == 0) st.ss_dr[static_cast<size_t>(t) * st.ss_dr_ld + b] = q;
+      }
     }
   }
 }

@@ -219,6 +219,8 @@ struct StepState {
 // before the next pass's embedding (the head computed B u itself).
 cudaError_t launch_finalize_draft(const StepState& st, int j, const HeadPrepArgs* prep, cudaStream_t s);
 cudaError_t launch_finalize_verify(const StepState& st, cudaStream_t s);
+// out_ids, n_committed and n_accepted to the caller's device buffers (each may be null).
+cudaError_t launch_copy_out(const StepState& st, int* ids, int* committed, int* accepted, cudaStream_t s);
 cudaError_t launch_finalize_ar(const StepState& st, cudaStream_t s);
 cudaError_t launch_finalize_prefill(const StepState& st, int seq, int n_tokens, int32_t* first_out,
                                     cudaStream_t s);

@@ -40,17 +40,19 @@ cudaError_t launch_embed(const EmbedArgs& a, cudaStream_t s) {
 // ---------------------------------------------------------------- head prep
 // grid (rows, ceil(r/4) or 1); block 128.  Every CTA computes the row's
 // 1/rms; CTA y == 0 logs u and hands the row to the verify stream; each CTA
-// computes four entries of B u (one warp each).
-template <typename T>
+// computes four entries of B u (one warp each).  NT bounds d / 128: at small d
+// the code for 64 tiles is mostly skipped, but fetched (11 us a launch at
+// d 256).
+template <typename T, int NT>
 __global__ void __launch_bounds__(128) head_prep_kernel(const HeadPrepArgs a) {
   __shared__ float red[kMaxTiles * 4];
   __shared__ float rstd_s;
-  __shared__ __align__(16) float us[kMaxTiles * kTileRows];   // u = x * rstd * gain
+  __shared__ __align__(16) float us[NT * kTileRows];   // u = x * rstd * gain
   griddep_launch();
   griddep_wait();
   const int row = blockIdx.x, grp = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  prep_row<T>(a, row, grp == 0, red, &rstd_s, us);
+  prep_row<T, NT>(a, row, grp == 0, red, &rstd_s, us);
   if (a.r > 0 && a.bu) {
     __syncthreads();
     const int j = grp * 4 + warp;
@@ -76,8 +78,11 @@ __global__ void __launch_bounds__(128) head_prep_kernel(const HeadPrepArgs a) {
 
 cudaError_t launch_head_prep(const HeadPrepArgs& a, cudaStream_t s) {
   dim3 grid(a.rows, (a.r > 0 && a.bu) ? (a.r + 3) / 4 : 1);
-  cudaError_t e = a.dtype == DVI_BF16 ? launch_pdl(head_prep_kernel<__nv_bfloat16>, grid, dim3(128), 0, s, a)
-                                      : launch_pdl(head_prep_kernel<float>, grid, dim3(128), 0, s, a);
+  const bool small = a.d <= 8 * kTileRows;
+  auto kern = a.dtype == DVI_BF16
+                  ? (small ? head_prep_kernel<__nv_bfloat16, 8> : head_prep_kernel<__nv_bfloat16, kMaxTiles>)
+                  : (small ? head_prep_kernel<float, 8> : head_prep_kernel<float, kMaxTiles>);
+  const cudaError_t e = launch_pdl(kern, grid, dim3(128), 0, s, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -163,6 +168,19 @@ cudaError_t launch_finalize_draft(const StepState& st, int j, const HeadPrepArgs
           : launch_pdl(finalize_draft_kernel<float>, dim3(1), dim3(128), smem, s, st, j, hp, on, stage);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
+// The step's outputs to the caller's buffers, one launch for the three.
+__global__ void __launch_bounds__(128) copy_out_kernel(const StepState st, int* ids, int* committed, int* accepted) {
+  for (int i = threadIdx.x; i < st.B * st.Kv && ids; i += 128) ids[i] = st.out_ids[i];
+  for (int i = threadIdx.x; i < st.B; i += 128) {
+    if (committed) committed[i] = st.n_committed[i];
+    if (accepted) accepted[i] = st.n_accepted[i];
+  }
+}
+cudaError_t launch_copy_out(const StepState& st, int* ids, int* committed, int* accepted, cudaStream_t s) {
+  copy_out_kernel<<<1, 128, 0, s>>>(st, ids, committed, accepted);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_finalize_verify(const StepState& st, cudaStream_t s) {
   return st.dtype == DVI_BF16 ? launch1(finalize_verify_kernel<__nv_bfloat16>, s, st)
                               : launch1(finalize_verify_kernel<float>, s, st);
