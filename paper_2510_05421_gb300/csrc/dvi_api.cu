@@ -275,20 +275,26 @@ size_t layout(dvi_ctx* c, char* base) {
   if (c->mk_sized) {
     MkArgs& a = c->mk;
     const size_t nqkv = static_cast<size_t>(c->Hq + 2 * c->Hkv) * c->hd;
-    a.xr = reinterpret_cast<float*>(take(sizeof(float) * 2 * B * d));
-    a.qkv = reinterpret_cast<float*>(take(sizeof(float) * B * nqkv));
     a.att = reinterpret_cast<float*>(take(sizeof(float) * B * c->Hq * a.P * c->hd));
     a.att_ml = reinterpret_cast<float*>(take(sizeof(float) * B * c->Hq * a.P * 2));
-    a.ao = reinterpret_cast<float*>(take(sizeof(float) * B * d));
-    a.hbuf = reinterpret_cast<float*>(take(sizeof(float) * B * c->F));
-    a.y = reinterpret_cast<float*>(take(sizeof(float) * B * d));
     a.bu_part = reinterpret_cast<float*>(take(sizeof(float) * c->n_sms * B * (r > 0 ? r : 1)));
+    // what is cleared before every launch, in one piece: the argmax keys, the
+    // tagged words, then the completion counters and the abort flag
+    const size_t keys_n = static_cast<size_t>((c->Kv * B + 1) / 2 * 2);
+    const size_t words = B * (nqkv + 2 * static_cast<size_t>(d) + c->F);
+    c->mk_sync_bytes = sizeof(uint64_t) * (keys_n + words) + sizeof(int) * (a.n_bound + 1);
     c->mk_sync = take(c->mk_sync_bytes);
+    uint64_t* w = reinterpret_cast<uint64_t*>(c->mk_sync);
+    a.keys = reinterpret_cast<unsigned long long*>(w);
+    if (w) {
+      w += keys_n;
+      a.qkv = w;
+      a.ao = a.qkv + B * nqkv;
+      a.y = a.ao + static_cast<size_t>(B) * d;
+      a.hbuf = a.y + static_cast<size_t>(B) * d;
+      a.ctr = reinterpret_cast<int*>(a.hbuf + static_cast<size_t>(B) * c->F);
+    }
     c->mk_maps_dev = reinterpret_cast<CUtensorMap*>(take(sizeof(CUtensorMap) * (7 * c->k + 3)));
-    a.keys = reinterpret_cast<unsigned long long*>(c->mk_sync);
-    a.ctr = c->mk_sync ? reinterpret_cast<int*>(static_cast<char*>(c->mk_sync) +
-                                                sizeof(unsigned long long) * c->Kv * B)
-                       : nullptr;
   }
   return align_up(off, 256);
 }
@@ -422,7 +428,6 @@ void size_mk(dvi_ctx* c) {
   for (int ns = 12; ns >= 4 && !a.n_stages; --ns)
     if (mk_smem_bytes(a, ns) <= 227 * 1024) a.n_stages = ns;
   if (!a.n_stages) return;
-  c->mk_sync_bytes = sizeof(unsigned long long) * c->Kv * c->B + sizeof(int) * (a.n_bound + 1);
   c->mk_sized = true;
 }
 

@@ -281,9 +281,10 @@ cudaError_t launch_update_full(const UpdateArgs& a, int n_sms, cudaStream_t s);
 // shallow passes of a decode step (Sec. 3.3): the k draft layers of every
 // draft pass with the drafter head, its argmax and the hand-off of h_k to the
 // verify rows (MK_DRAFT), or the k shallow layers of one greedy AR step with
-// the hand-off to the AR rows (MK_AR).  Phases (QKV, attention, O, gate/up,
-// down, head) meet at release/acquire completion counters, one per phase
-// boundary, with bounded polls.  bf16 weights only; at most kMkMaxRows
+// the hand-off to the AR rows (MK_AR).  Projection rows pass from
+// phase to phase (QKV, attention, O, gate/up, down) as tagged 64-bit words;
+// the attention, B u and argmax results meet at release/acquire completion
+// counters.  All polls are bounded.  bf16 weights only; at most kMkMaxRows
 // sequences.
 constexpr int kMkMaxLayers = 16;
 constexpr int kMkMaxRows = 2;
@@ -314,13 +315,13 @@ struct MkArgs {
   void* log_u; size_t log_plane; const int* log_step; int log_cap_steps; int log_enabled;
   float* zlog;
   // scratch
-  float* xr;             // [2][B][d] residual stream (double buffered)
-  float* qkv;            // [B][(H_q + 2 H_kv) hd] projections before RoPE
+  // (qkv, ao, hbuf and y: tagged words {f32, tag}, zero before the launch)
+  uint64_t* qkv;         // [B][(H_q + 2 H_kv) hd] projections before RoPE
   float* att;            // [B][H_q][P][hd] attention partials: o
   float* att_ml;         // [B][H_q][P][2] their (max, sum)
-  float* ao;             // [B][d] output projection
-  float* hbuf;           // [B][F] SwiGLU
-  float* y;              // [B][d] down projection
+  uint64_t* ao;          // [B][d] output projection
+  uint64_t* hbuf;        // [B][F] SwiGLU
+  uint64_t* y;           // [B][d] down projection
   float* bu_part;        // [n_ctas][r] partial B u
   unsigned long long* keys;   // [Kv][B] argmax keys, zero before the launch
   int* ctr;              // [n_bound + 1] zero before the launch

@@ -6,21 +6,24 @@
 //       QKV -> attention -> O -> gate/up (SwiGLU) -> down
 //     then the hand-off of h_{k} to the verify rows and, for j < K, the
 //     drafter head z = W^S u + gamma A (B u) with its argmax (the next draft).
-// A phase ends with a completion counter: each CTA adds 1 with release
-// semantics after its global writes, and the next phase polls the count with
-// acquire semantics (bounded; a timeout sets DVI_DEV_TIMEOUT and an abort
-// flag that ends every CTA's loop).
+// The projections' outputs travel to the next phase as tagged words, which
+// the readers poll; the attention's partials, B u and the argmax meet at
+// completion counters: each CTA adds 1 with release semantics after its global
+// writes, and the next phase polls the count with acquire semantics.  Every
+// poll is bounded; a timeout sets DVI_DEV_TIMEOUT and an abort flag that ends
+// every CTA's loop.
 //
 // Projections are row-split: each CTA owns a contiguous range of 8-row groups
 // of a weight matrix's output rows with the whole K, so a row's dot product
 // is finished inside one CTA and no partial sums cross CTAs.  The decode rows
-// are few (at most kMkMaxRows), so every CTA rebuilds the small input vector
-// of a phase itself (residual adds, RMSNorm statistics, attention combine)
-// from the previous phase's outputs instead of waiting for one owner.
+// are few (at most kMkMaxRows), so every CTA keeps the residual rows in its
+// shared memory and rebuilds the small input vector of a phase itself
+// (residual adds, RMSNorm statistics, attention combine) from the previous
+// phase's outputs instead of waiting for one owner.
 // Warp 8 streams the CTA's weight tiles (8 rows x 64 columns, 128-byte
 // swizzle, 16 per 16 KB stage) and the attention's cached K/V rows through a
 // ring of stages, running ahead across phase boundaries, so HBM keeps
-// streaming while the CTAs meet at a counter.  Warps 0-7 compute: each warp
+// streaming while the CTAs meet.  Warps 0-7 compute: each warp
 // takes 128 of a stage's 1024 columns and multiplies the 8 weight rows
 // (B operand, by ldmatrix) with the activations (A operand: rows are the bf16
 // hi and lo halves of each decode row, the rest zero) on the warp tensor
@@ -147,7 +150,7 @@ size_t mk_smem_bytes(const MkArgs& a, int n_stages) { return mk_layout(a, n_stag
 int mk_bounds(const MkArgs& a) {
   const int npass = a.mode == MK_DRAFT ? a.Kv : 1;
   const int heads = a.mode == MK_DRAFT ? a.K : 0;
-  return npass * 5 * a.k + 2 * heads;
+  return npass * a.k + 2 * heads;   // the attention of every layer instance; B u and the argmax of every head
 }
 
 int mk_rows_max(const MkArgs& a, int n) {
@@ -231,6 +234,78 @@ __device__ __forceinline__ void mk_abort(const MkArgs& a) {
   *abort_flag = 1;
 }
 
+// ------------------------------------------------------------------ tagged words
+// What one phase hands to the next by value (projection rows) travels as
+// 64-bit words, the f32 value below a tag that names the layer instance (j k +
+// l + 1; the words are cleared before the launch).  One 64-bit store or load
+// is a single access, so a reader that sees the tag has the value, with no
+// counter, release or fence between: the readers poll the words themselves.
+// Only the attention's partials still meet at a counter, and since every CTA
+// passes that one in every layer, a word is never overwritten before its last
+// reader is done: a CTA that has reached layer l's counter has read all that
+// layers before l (and layer l's QKV) wrote.
+// What this saves is the counter's chain at a phase boundary: stores, fence,
+// CTA barrier, atomic, poll, CTA barrier, then the loads it guarded -- three
+// trips to L2 instead of one.  Draft phase 1442 -> 1323 us (1B workload, 200
+// boundaries, 160 of them now words), 1077 -> 1042 (7B, 50 and 40; HBM-bound
+// between them).  The words are twice the bytes of f32 rows, all from L2.
+// Backing off between polls (__nanosleep(100)) loses it all: 1531 us.
+__device__ __forceinline__ void ll_store(uint64_t* p, float v, uint32_t tag) {
+  const uint64_t w = (static_cast<uint64_t>(tag) << 32) | __float_as_uint(v);
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ uint64_t ll_load(const uint64_t* p) {
+  uint64_t w;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  return w;
+}
+__device__ __forceinline__ void ll_load2(const uint64_t* p, uint64_t& a, uint64_t& b) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+__device__ __forceinline__ uint32_t ll_tag(uint64_t w) { return static_cast<uint32_t>(w >> 32); }
+__device__ __forceinline__ float ll_val(uint64_t w) { return __uint_as_float(static_cast<uint32_t>(w)); }
+// A word that is not wanted: it counts as arrived and is never loaded.
+__device__ __forceinline__ uint64_t ll_skip(uint32_t tag) { return static_cast<uint64_t>(tag) << 32; }
+// Loads a word, or a pair, again while its tag is not `tag` (a polling thread
+// asks only for what it still misses; the loads of one round are independent).
+__device__ __forceinline__ void ll_again(uint64_t& w, const uint64_t* p, uint32_t tag) {
+  if (ll_tag(w) != tag) w = ll_load(p);
+}
+__device__ __forceinline__ void ll_again2(uint64_t (&w)[2], const uint64_t* p, uint32_t tag) {
+  if (ll_tag(w[0]) != tag || ll_tag(w[1]) != tag) ll_load2(p, w[0], w[1]);
+}
+// Repeats `load` (a round of a thread's loads, then the check of their tags)
+// until it succeeds; bounded like mk_wait.
+template <typename F>
+__device__ __forceinline__ bool ll_spin(const MkArgs& a, F load) {
+  uint64_t t0 = 0;
+  for (uint32_t it = 1; !load(); ++it) {
+    if ((it & 63u) != 0) continue;
+    volatile int* abort_flag = a.ctr + a.n_bound;
+    if (*abort_flag) return false;
+    if (t0 == 0) t0 = global_ns();
+    if (global_ns() - t0 > kWaitLimitNs) {
+      flag_status(a.status, DVI_DEV_TIMEOUT);
+      *abort_flag = 1;
+      return false;
+    }
+  }
+  return true;
+}
+// The compute barrier, true when any thread's wait has failed.
+__device__ __forceinline__ bool cbar_any(bool failed) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %1, 0;\n\t"
+      "barrier.cta.red.or.pred q, %2, %3, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(failed ? 1u : 0u), "r"(kMkBar), "r"(kMkCompute)
+      : "memory");
+  return r != 0;
+}
+
 // Bounded wait on an mbarrier phase that also gives up when the launch is
 // aborting (checked every 256 polls).
 __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t parity, const MkArgs& a) {
@@ -246,6 +321,31 @@ __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t parity, 
       return false;
     }
   }
+}
+
+// act[m][i] = x * rstd[m] * g[i]
+// (the gains are loaded eight per thread at a time)
+__device__ __forceinline__ void mk_scale(const MkArgs& a, float* act, const float* rstd, const float* __restrict__ g) {
+  for (int i0 = threadIdx.x; i0 < a.d; i0 += 8 * kMkCompute) {
+    float gv[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * kMkCompute;
+      gv[u] = i < a.d ? __ldg(g + i) : 0.f;
+    }
+    for (int m = 0; m < a.B; ++m) {
+      const float r = rstd[m];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = i0 + u * kMkCompute;
+        if (i < a.d) {
+          const size_t o = static_cast<size_t>(m) * a.d + i;
+          act[o] = act[o] * r * gv[u];
+        }
+      }
+    }
+  }
+  cbar();
 }
 
 }  // namespace
@@ -333,42 +433,68 @@ __device__ __forceinline__ void gemv_finish(float* wacc, int rows_max, int nrows
 }
 
 // The A operand of a projection over K columns: plane 2m (hi) and 2m + 1
-// (lo) of row m of src (row stride ld), as bf16 pairs (columns 2w, 2w + 1 in
-// word w of the plane), zero from K to the end of the last 1024-column
-// chunk.  `global`: src is in global memory, written by other CTAs in the
-// previous phase (four loads per thread in flight).
+// (lo) of row m, as bf16 pairs (columns 2w, 2w + 1 in word w of the plane),
+// zero from K to the end of the last 1024-column chunk.  From f32 rows in
+// shared memory (row stride ld), times rstd[m] * g when g is set.
 template <int M>
-__device__ __forceinline__ void mk_pack(uint32_t* xw, int plane, const float* src, int K, int ld, bool global) {
+__device__ __forceinline__ void mk_pack(uint32_t* xw, int plane, const float* src, int K, int ld,
+                                        const float* rstd = nullptr, const float* __restrict__ g = nullptr) {
   const int nw = mk_chunks(K) * kMkChunk / 2, kw = K / 2, pw = plane / 2;
-  for (int w0 = threadIdx.x; w0 < nw; w0 += 4 * kMkCompute) {
-    float2 v[4][M];
+  for (int w = threadIdx.x; w < nw; w += kMkCompute) {
+    const float2 gv = g && w < kw ? __ldg(reinterpret_cast<const float2*>(g) + w) : make_float2(1.f, 1.f);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int w = w0 + u * kMkCompute;
-#pragma unroll
-      for (int m = 0; m < M; ++m) {
-        v[u][m] = make_float2(0.f, 0.f);
-        if (w < kw) {
-          const float2* p = reinterpret_cast<const float2*>(src + static_cast<size_t>(m) * ld) + w;
-          v[u][m] = global ? __ldcg(p) : *p;
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int w = w0 + u * kMkCompute;
-      if (w < nw) {
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-          uint32_t hi, lo;
-          split_bf16x2(v[u][m].x, v[u][m].y, hi, lo);
-          xw[(2 * m) * pw + w] = hi;
-          xw[(2 * m + 1) * pw + w] = lo;
-        }
-      }
+    for (int m = 0; m < M; ++m) {
+      float2 v = make_float2(0.f, 0.f);
+      if (w < kw) v = reinterpret_cast<const float2*>(src + static_cast<size_t>(m) * ld)[w];
+      if (g) v = make_float2(v.x * rstd[m] * gv.x, v.y * rstd[m] * gv.y);
+      uint32_t hi, lo;
+      split_bf16x2(v.x, v.y, hi, lo);
+      xw[(2 * m) * pw + w] = hi;
+      xw[(2 * m + 1) * pw + w] = lo;
     }
   }
   cbar();
+}
+// The same from tagged rows of K words (the down projection's input), eight
+// words per thread and row in flight.  False when the launch is aborting.
+template <int M>
+__device__ __forceinline__ bool mk_pack_ll(const MkArgs& a, uint32_t* xw, int plane, const uint64_t* src, int K,
+                                           uint32_t tag) {
+  const int nw = mk_chunks(K) * kMkChunk / 2, kw = K / 2, pw = plane / 2;
+  bool ok = true;
+  for (int w0 = threadIdx.x; w0 < nw && ok; w0 += 4 * kMkCompute) {
+    uint64_t v[4][M][2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int m = 0; m < M; ++m) v[u][m][0] = v[u][m][1] = w0 + u * kMkCompute < kw ? 0ull : ll_skip(tag);
+    ok = ll_spin(a, [&]() {
+      bool good = true;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+          ll_again2(v[u][m], src + static_cast<size_t>(m) * K + 2 * (w0 + u * kMkCompute), tag);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int m = 0; m < M; ++m) good = good && ll_tag(v[u][m][0]) == tag && ll_tag(v[u][m][1]) == tag;
+      return good;
+    });
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int w = w0 + u * kMkCompute;
+      if (w >= nw) continue;
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        uint32_t hi = 0u, lo = 0u;
+        if (w < kw) split_bf16x2(ll_val(v[u][m][0]), ll_val(v[u][m][1]), hi, lo);
+        xw[(2 * m) * pw + w] = hi;
+        xw[(2 * m + 1) * pw + w] = lo;
+      }
+    }
+  }
+  return !cbar_any(!ok);
 }
 
 // ------------------------------------------------------------------ phase geometry
@@ -396,7 +522,8 @@ __device__ __forceinline__ const CUtensorMap* qkv_group(const MkArgs& a, int l, 
 // its unit about 0.4 us.
 // Draft phase of the 1B workload (5 passes of 8 layers, 512 positions) 2.08
 // -> 1.41 ms and of the 7B one (5 x 2, 1024) 1.14 -> 1.06 ms, with the O
-// phase's combine and the compute warps' registers.
+// phase's combine and the compute warps' registers (1.32 and 1.04 ms with
+// the tagged words).
 constexpr int kMkUnitChunks = 2;
 __device__ __forceinline__ int att_chunks(int pos, int hd) { return pos / (kMkStageElems / hd) + 1; }
 __device__ __forceinline__ int att_parts(const MkArgs& a, int pos) {
@@ -524,36 +651,40 @@ __device__ void mk_producer(const MkArgs& a, Ring& r, int c, int n) {
 }
 
 // ------------------------------------------------------------------ prologues
-// act[m][0..d) = the raw residual of row m: xa[m] + xb[m] (written by other
-// CTAs in earlier phases) or the embedding of tok[m]; `writer` also stores it
-// in xr_out.
-// (Loads are issued eight per thread at a time before any result is stored.)
-__device__ __forceinline__ void mk_residual(const MkArgs& a, float* act, const float* __restrict__ xa,
-                                            const float* __restrict__ xb, const int* tok, float* xr_out,
-                                            bool writer) {
-  const int d = a.d;
+// The residual rows live in every CTA's shared memory (act[m][0..d)): each
+// CTA adds what a projection hands over itself.
+// act[m] = the embedding of tok[m].
+__device__ __forceinline__ void mk_embed(const MkArgs& a, float* act, const int* tok) {
   for (int m = 0; m < a.B; ++m) {
-    const __nv_bfloat16* e =
-        tok ? static_cast<const __nv_bfloat16*>(a.embed) + static_cast<size_t>(tok[m]) * d : nullptr;
-    const size_t base = static_cast<size_t>(m) * d;
-    for (int i0 = threadIdx.x; i0 < d; i0 += 8 * kMkCompute) {
-      float v[8];
+    const __nv_bfloat16* e = static_cast<const __nv_bfloat16*>(a.embed) + static_cast<size_t>(tok[m]) * a.d;
+    for (int i = threadIdx.x; i < a.d; i += kMkCompute)
+      act[static_cast<size_t>(m) * a.d + i] = __bfloat162float(e[i]);
+  }
+}
+// act[m] += the tagged rows y (eight words per thread in flight).  False when
+// the launch is aborting.
+__device__ __forceinline__ bool mk_add(const MkArgs& a, float* act, const uint64_t* y, uint32_t tag) {
+  bool ok = true;
+  const int n = a.B * a.d;
+  for (int i0 = threadIdx.x; i0 < n && ok; i0 += 8 * kMkCompute) {
+    uint64_t v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int i = i0 + u * kMkCompute;
-        v[u] = 0.f;
-        if (i < d) v[u] = e ? __bfloat162float(e[i]) : __ldcg(xa + base + i) + __ldcg(xb + base + i);
-      }
+    for (int u = 0; u < 8; ++u) v[u] = i0 + u * kMkCompute < n ? 0ull : ll_skip(tag);
+    ok = ll_spin(a, [&]() {
+      bool good = true;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int i = i0 + u * kMkCompute;
-        if (i < d) {
-          act[base + i] = v[u];
-          if (writer) xr_out[base + i] = v[u];
-        }
-      }
+      for (int u = 0; u < 8; ++u) ll_again(v[u], y + i0 + u * kMkCompute, tag);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) good = good && ll_tag(v[u]) == tag;
+      return good;
+    });
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * kMkCompute;
+      if (i < n) act[i] += ll_val(v[u]);
     }
   }
+  return !cbar_any(!ok);
 }
 
 // Per-128-feature sums of squares of the act rows (tsum[m][t]) and 1/rms.
@@ -582,31 +713,6 @@ __device__ __forceinline__ void mk_rms(const MkArgs& a, const float* act, float*
   cbar();
 }
 
-// act[m][i] = x * rstd[m] * g[i]
-// (the gains are loaded eight per thread at a time)
-__device__ __forceinline__ void mk_scale(const MkArgs& a, float* act, const float* rstd, const float* __restrict__ g) {
-  for (int i0 = threadIdx.x; i0 < a.d; i0 += 8 * kMkCompute) {
-    float gv[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * kMkCompute;
-      gv[u] = i < a.d ? __ldg(g + i) : 0.f;
-    }
-    for (int m = 0; m < a.B; ++m) {
-      const float r = rstd[m];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int i = i0 + u * kMkCompute;
-        if (i < a.d) {
-          const size_t o = static_cast<size_t>(m) * a.d + i;
-          act[o] = act[o] * r * gv[u];
-        }
-      }
-    }
-  }
-  cbar();
-}
-
 }  // namespace
 }  // namespace dvi
 
@@ -614,38 +720,63 @@ namespace dvi {
 namespace {
 
 // The normed input of a projection over d columns in one pass (d <= 4096):
-// x = xa + xb (or the embedding of tok), stored to xr_out by `writer`; the
-// per-128-feature sums of squares and 1/rms; the A planes of x * rstd * g.  Thread tid takes the column pairs tid + 256 e, whose loads
-// (x and gain) are all issued before any is used; a warp's 32 pairs are half
-// a 128-column tile, so the tile sums are two warp sums (hs[m][tile][half]).
+// the residual act += y (tagged rows; or the embedding of tok), the
+// per-128-feature sums of squares and 1/rms; the A planes of x * rstd * g.
+// Thread tid takes the column pairs tid + 256 e, whose loads (y and gain) are
+// all issued before any is used; a warp's 32 pairs are half a 128-column
+// tile, so the tile sums are two warp sums (hs[m][tile][half]).  False when
+// the launch is aborting.
 constexpr int kMkPairs = 8;   // column pairs per thread: d <= 512 * kMkPairs
 template <int M>
-__device__ __forceinline__ void mk_norm_pack(const MkArgs& a, const float* __restrict__ xa,
-                                             const float* __restrict__ xb, const int* tok, float* xr_out,
-                                             bool writer, const float* __restrict__ g, uint32_t* xw, int plane,
+__device__ __forceinline__ bool mk_norm_pack(const MkArgs& a, float* act, const uint64_t* y, uint32_t tag,
+                                             const int* tok, const float* __restrict__ g, uint32_t* xw, int plane,
                                              float* hs) {
   const int d = a.d, np = d / 2, nt = d / 128, pw = plane / 2;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float2 x[M][kMkPairs], gv[kMkPairs];
 #pragma unroll
   for (int e = 0; e < kMkPairs; ++e) {
-    const int p = tid + e * kMkCompute;
-    gv[e] = make_float2(0.f, 0.f);
+    const int p = min(tid + e * kMkCompute, np - 1);
+    gv[e] = __ldg(reinterpret_cast<const float2*>(g) + p);
+  }
+  bool ok = true;
+  if (tok) {
 #pragma unroll
-    for (int m = 0; m < M; ++m) x[m][e] = make_float2(0.f, 0.f);
-    if (p < np) {
-      gv[e] = __ldg(reinterpret_cast<const float2*>(g) + p);
+    for (int e = 0; e < kMkPairs; ++e) {
+      const int p = min(tid + e * kMkCompute, np - 1);
 #pragma unroll
       for (int m = 0; m < M; ++m) {
-        if (tok) {
-          const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const __nv_bfloat16*>(a.embed) +
-                                                                      static_cast<size_t>(tok[m]) * d) + p);
-          x[m][e] = make_float2(bf16_lo(w), bf16_hi(w));
-        } else {
-          const float2 u = __ldcg(reinterpret_cast<const float2*>(xa + static_cast<size_t>(m) * d) + p);
-          const float2 v = __ldcg(reinterpret_cast<const float2*>(xb + static_cast<size_t>(m) * d) + p);
-          x[m][e] = make_float2(u.x + v.x, u.y + v.y);
-        }
+        const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const __nv_bfloat16*>(a.embed) +
+                                                                    static_cast<size_t>(tok[m]) * d) + p);
+        x[m][e] = make_float2(bf16_lo(w), bf16_hi(w));
+      }
+    }
+  } else {
+    uint64_t v[M][kMkPairs][2];
+#pragma unroll
+    for (int e = 0; e < kMkPairs; ++e)
+#pragma unroll
+      for (int m = 0; m < M; ++m) v[m][e][0] = v[m][e][1] = tid + e * kMkCompute < np ? 0ull : ll_skip(tag);
+    ok = ll_spin(a, [&]() {
+      bool good = true;
+#pragma unroll
+      for (int e = 0; e < kMkPairs; ++e)
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+          ll_again2(v[m][e], y + static_cast<size_t>(m) * d + 2 * (tid + e * kMkCompute), tag);
+#pragma unroll
+      for (int e = 0; e < kMkPairs; ++e)
+#pragma unroll
+        for (int m = 0; m < M; ++m) good = good && ll_tag(v[m][e][0]) == tag && ll_tag(v[m][e][1]) == tag;
+      return good;
+    });
+#pragma unroll
+    for (int e = 0; e < kMkPairs; ++e) {
+      const int p = min(tid + e * kMkCompute, np - 1);
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const float2 r = reinterpret_cast<const float2*>(act + static_cast<size_t>(m) * d)[p];
+        x[m][e] = make_float2(r.x + ll_val(v[m][e][0]), r.y + ll_val(v[m][e][1]));
       }
     }
   }
@@ -655,13 +786,13 @@ __device__ __forceinline__ void mk_norm_pack(const MkArgs& a, const float* __res
     if (p < np) {
 #pragma unroll
       for (int m = 0; m < M; ++m) {
-        if (writer) reinterpret_cast<float2*>(xr_out + static_cast<size_t>(m) * d)[p] = x[m][e];
+        reinterpret_cast<float2*>(act + static_cast<size_t>(m) * d)[p] = x[m][e];
         const float sq = warp_sum(fmaf(x[m][e].x, x[m][e].x, x[m][e].y * x[m][e].y));
         if (lane == 0) hs[(m * nt + (e * kMkCompute + warp * 32) / 64) * 2 + (warp & 1)] = sq;
       }
     }
   }
-  cbar();
+  if (cbar_any(!ok)) return false;
   // every warp sums the row's tiles itself, one a lane (nt <= 32): no
   // serial chain over the tiles and no second barrier
   float rs[M];
@@ -690,6 +821,7 @@ __device__ __forceinline__ void mk_norm_pack(const MkArgs& a, const float* __res
 #pragma unroll
     for (int q = 0; q < 2 * M; ++q) xw[q * pw + w] = 0u;
   cbar();
+  return true;
 }
 
 // ------------------------------------------------------------------ attention
@@ -757,7 +889,8 @@ __device__ __forceinline__ uint32_t kv_mask(uint32_t v, int p, int cn) {
 // (compact code: the phase runs after the projections' code has filled the
 // instruction cache).
 template <int HD, int G>
-__device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& ring, uint8_t* att_sm) {
+__device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& ring, uint8_t* att_sm, float* raw,
+                             uint32_t tag) {
   constexpr int CP = kMkStageElems / HD;   // positions per stage
   constexpr int PW = CP / kMkWarps;        // positions per warp and stage
   constexpr int NT = PW / 8;               // score n-tiles per warp
@@ -773,15 +906,40 @@ __device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& rin
   __nv_bfloat16* kn = reinterpret_cast<__nv_bfloat16*>(qf + KS * QL);   // [HD]
   __nv_bfloat16* vn = kn + HD;
 
-  const float* qrow = a.qkv + static_cast<size_t>(u.b) * (a.Hq + 2 * a.Hkv) * HD;
+  // the unit's rows before RoPE, G queries, key, value, into shared memory
+  {
+    const uint64_t* row = a.qkv + static_cast<size_t>(u.b) * (a.Hq + 2 * a.Hkv) * HD;
+    constexpr int N = (G + 2) * HD, E = (N + kMkCompute - 1) / kMkCompute;
+    uint64_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = tid + e * kMkCompute < N ? 0ull : ll_skip(tag);
+    const bool got = ll_spin(a, [&]() {
+      bool good = true;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int i = tid + e * kMkCompute;
+        const int at = i < G * HD ? u.kvh * G * HD + i
+                                  : (i < (G + 1) * HD ? (a.Hq + u.kvh) * HD + i - G * HD
+                                                      : (a.Hq + a.Hkv + u.kvh) * HD + i - (G + 1) * HD);
+        ll_again(v[e], row + at, tag);
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) good = good && ll_tag(v[e]) == tag;
+      return good;
+    });
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (tid + e * kMkCompute < N) raw[tid + e * kMkCompute] = ll_val(v[e]);
+    if (cbar_any(!got)) return false;
+  }
   const bool pos_ok = u.pos < a.max_len;
   const int rp = pos_ok ? u.pos : a.max_len - 1;
   const float2* rope = a.rope + static_cast<size_t>(rp) * half;
   const float qscale = kLog2e * rsqrtf(static_cast<float>(HD));
-  // dimension dim of head row h of this row's q | k after RoPE
+  // dimension dim of row h (a query head of the group; G: the key) after RoPE
   auto rot = [&](int h, int dim) {
-    const float* x = qrow + static_cast<size_t>(h) * HD;
-    const float v = __ldcg(x + dim), vp = __ldcg(x + (dim < half ? dim + half : dim - half));
+    const float* x = raw + h * HD;
+    const float v = x[dim], vp = x[dim < half ? dim + half : dim - half];
     const float2 cs = rope[dim % half];
     return dim < half ? v * cs.x - vp * cs.y : v * cs.x + vp * cs.y;
   };
@@ -793,7 +951,7 @@ __device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& rin
     for (int r = 0; r < 2; ++r) {
       const int row = gg + 8 * r, hq = row >> 1;
       if (hq < G) {
-        const int h = u.kvh * G + hq, d0 = 16 * ks + 2 * cc;
+        const int h = hq, d0 = 16 * ks + 2 * cc;
         uint32_t hi0, lo0, hi1, lo1;
         split_bf16x2(rot(h, d0) * qscale, rot(h, d0 + 1) * qscale, hi0, lo0);
         split_bf16x2(rot(h, d0 + 8) * qscale, rot(h, d0 + 9) * qscale, hi1, lo1);
@@ -804,8 +962,8 @@ __device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& rin
     qf[i] = make_uint4(f[0], f[1], f[2], f[3]);
   }
   for (int dim = tid; dim < HD; dim += kMkCompute) {
-    kn[dim] = __float2bfloat16_rn(rot(a.Hq + u.kvh, dim));
-    vn[dim] = __float2bfloat16_rn(__ldcg(qrow + static_cast<size_t>(a.Hq + a.Hkv + u.kvh) * HD + dim));
+    kn[dim] = __float2bfloat16_rn(rot(G, dim));
+    vn[dim] = __float2bfloat16_rn(raw[(G + 1) * HD + dim]);
   }
   cbar();
   // the newest position into the cache (the unit whose range ends at pos)
@@ -994,15 +1152,15 @@ __device__ bool mk_attention(const MkArgs& a, int l, const AttUnit& u, Ring& rin
 // The unit's attention for the GQA group size of the model (1, 2, 4 or 8).
 template <int HD>
 __device__ __forceinline__ bool mk_attention_any(const MkArgs& a, int l, const AttUnit& u, Ring& ring,
-                                                 uint8_t* att_sm) {
+                                                 uint8_t* att_sm, float* raw, uint32_t tag) {
   switch (a.Hq / a.Hkv) {
-    case 1: return mk_attention<HD, 1>(a, l, u, ring, att_sm);
-    case 2: return mk_attention<HD, 2>(a, l, u, ring, att_sm);
-    case 4: return mk_attention<HD, 4>(a, l, u, ring, att_sm);
+    case 1: return mk_attention<HD, 1>(a, l, u, ring, att_sm, raw, tag);
+    case 2: return mk_attention<HD, 2>(a, l, u, ring, att_sm, raw, tag);
+    case 4: return mk_attention<HD, 4>(a, l, u, ring, att_sm, raw, tag);
     default:
       // a group of 8 at head_dim 128 (o^T in 64 registers a lane) is not
       // given to this kernel
-      if constexpr (HD == 64) return mk_attention<HD, 8>(a, l, u, ring, att_sm);
+      if constexpr (HD == 64) return mk_attention<HD, 8>(a, l, u, ring, att_sm, raw, tag);
       return false;
   }
 }
@@ -1129,10 +1287,8 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
   part_range(mk_groups(a.F), c, n, f0, f1);
   part_range(mk_groups(a.V), c, n, v0, v1);
   part_range(d, c, n, h0, h1);
-  float* xr[2] = {a.xr, a.xr + static_cast<size_t>(M) * d};
   int bn = 0;    // next completion counter
-  int bw = -1;   // counter the next phase waits for
-  int cur = 0;   // xr slot that holds the residual
+  int bw = -1;   // counter of the previous pass's head, if any
   for (int j = 0; j < npass; ++j) {
     const bool head = a.mode == MK_DRAFT && j < K;
     const AttUnit u = att_unit(a, j, c);
@@ -1141,9 +1297,10 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
     for (int m = 0; m < M; ++m) np[m] = att_parts(a, a.lens[m] + j);
     for (int l = 0; l < a.k; ++l) {
       const MkLayerW& w = a.layer[l];
+      const uint32_t tag = static_cast<uint32_t>(j * a.k + l + 1);
       // ---------------- QKV
-      if (bw >= 0 && !mk_wait(a, bw, flag_s)) return;
       if (l == 0) {
+        if (bw >= 0 && !mk_wait(a, bw, flag_s)) return;
         if (tid < M) {
           int t;
           if (j == 0) {
@@ -1164,54 +1321,43 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
         cbar();
       }
       if (fused) {
-        mk_norm_pack<M>(a, xr[cur], a.y, l == 0 ? tok : nullptr, xr[cur ^ 1], c == 0, w.g_attn, xw, plane, hs);
+        if (!mk_norm_pack<M>(a, act, a.y, tag - 1, l == 0 ? tok : nullptr, w.g_attn, xw, plane, hs)) return;
       } else {
-        if (l == 0) mk_residual(a, act, nullptr, nullptr, tok, xr[cur ^ 1], c == 0);
-        else mk_residual(a, act, xr[cur], a.y, nullptr, xr[cur ^ 1], c == 0);
+        if (l == 0) mk_embed(a, act, tok);
+        else if (!mk_add(a, act, a.y, tag - 1)) return;
         mk_rms(a, act, tsum, rstd);
-        mk_scale(a, act, rstd, w.g_attn);
-        mk_pack<M>(xw, plane, act, d, d, false);
+        mk_pack<M>(xw, plane, act, d, d, rstd, w.g_attn);
       }
-      cur ^= 1;
       if (!gemv_groups<M>(ring, d, q0, q1, xa, plane, wacc, rows_max, a.status)) {
         mk_abort(a);
         return;
       }
       gemv_finish<M>(wacc, rows_max, (q1 - q0) * kMkGroup,
-                     [&](int rl, int m, float v) { a.qkv[m * nqkv + q0 * kMkGroup + rl] = v; });
-      mk_signal(a, bn);
-      bw = bn++;
+                     [&](int rl, int m, float v) { ll_store(a.qkv + m * nqkv + q0 * kMkGroup + rl, v, tag); });
       // ---------------- attention
-      if (!mk_wait(a, bw, flag_s)) return;
-      if (u.on && !mk_attention_any<HD>(a, l, u, ring, att_sm)) {
+      if (u.on && !mk_attention_any<HD>(a, l, u, ring, att_sm, reinterpret_cast<float*>(xw), tag)) {
         mk_abort(a);
         return;
       }
       mk_signal(a, bn);
-      bw = bn++;
       // ---------------- O
-      if (!mk_wait(a, bw, flag_s)) return;
+      if (!mk_wait(a, bn++, flag_s)) return;
       mk_att_combine<HD, M>(a, np, xw, plane, reinterpret_cast<float*>(att_sm));
       if (!gemv_groups<M>(ring, nq, o0, o1, xa, plane, wacc, rows_max, a.status)) {
         mk_abort(a);
         return;
       }
       gemv_finish<M>(wacc, rows_max, (o1 - o0) * kMkGroup, [&](int rl, int m, float v) {
-        a.ao[static_cast<size_t>(m) * d + o0 * kMkGroup + rl] = v;
+        ll_store(a.ao + static_cast<size_t>(m) * d + o0 * kMkGroup + rl, v, tag);
       });
-      mk_signal(a, bn);
-      bw = bn++;
       // ---------------- gate / up
-      if (!mk_wait(a, bw, flag_s)) return;
       if (fused) {
-        mk_norm_pack<M>(a, xr[cur], a.ao, nullptr, xr[cur ^ 1], c == 0, w.g_ffn, xw, plane, hs);
+        if (!mk_norm_pack<M>(a, act, a.ao, tag, nullptr, w.g_ffn, xw, plane, hs)) return;
       } else {
-        mk_residual(a, act, xr[cur], a.ao, nullptr, xr[cur ^ 1], c == 0);
+        if (!mk_add(a, act, a.ao, tag)) return;
         mk_rms(a, act, tsum, rstd);
-        mk_scale(a, act, rstd, w.g_ffn);
-        mk_pack<M>(xw, plane, act, d, d, false);
+        mk_pack<M>(xw, plane, act, d, d, rstd, w.g_ffn);
       }
-      cur ^= 1;
       if (!gemv_groups<M>(ring, d, f0, f1, xa, plane, wacc, rows_max, a.status)) {
         mk_abort(a);
         return;
@@ -1223,26 +1369,20 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
       }
       gemv_finish<M>(wacc, rows_max, (f1 - f0) * kMkGroup, [&](int rl, int m, float v) {
         const float g = gbuf[rl * M + m];   // written by this thread in the gate's finish
-        a.hbuf[static_cast<size_t>(m) * a.F + f0 * kMkGroup + rl] = g / (1.f + expf(-g)) * v;
+        ll_store(a.hbuf + static_cast<size_t>(m) * a.F + f0 * kMkGroup + rl, g / (1.f + expf(-g)) * v, tag);
       });
-      mk_signal(a, bn);
-      bw = bn++;
       // ---------------- down
-      if (!mk_wait(a, bw, flag_s)) return;
-      mk_pack<M>(xw, plane, a.hbuf, a.F, a.F, true);
+      if (!mk_pack_ll<M>(a, xw, plane, a.hbuf, a.F, tag)) return;
       if (!gemv_groups<M>(ring, a.F, o0, o1, xa, plane, wacc, rows_max, a.status)) {
         mk_abort(a);
         return;
       }
       gemv_finish<M>(wacc, rows_max, (o1 - o0) * kMkGroup, [&](int rl, int m, float v) {
-        a.y[static_cast<size_t>(m) * d + o0 * kMkGroup + rl] = v;
+        ll_store(a.y + static_cast<size_t>(m) * d + o0 * kMkGroup + rl, v, tag);
       });
-      mk_signal(a, bn);
-      bw = bn++;
     }
     // ---------------- h_k: hand-off to the verify (or AR) rows, drafter head
-    if (!mk_wait(a, bw, flag_s)) return;
-    mk_residual(a, act, xr[cur], a.y, nullptr, nullptr, false);
+    if (!mk_add(a, act, a.y, static_cast<uint32_t>((j + 1) * a.k))) return;
     mk_rms(a, act, tsum, rstd);
     for (int m = 0; m < M; ++m) {
       const size_t row = static_cast<size_t>(m) * a.copy_row_stride + (a.mode == MK_DRAFT ? j : 0);
@@ -1284,7 +1424,7 @@ __device__ void mk_compute(const MkArgs& a, Ring& ring, const MkLayout& L, uint8
       mk_signal(a, bn);
       bu_bound = bn++;
     }
-    mk_pack<M>(xw, plane, act, d, d, false);
+    mk_pack<M>(xw, plane, act, d, d);
     if (!gemv_groups<M>(ring, d, v0, v1, xa, plane, wacc, rows_max, a.status)) {
       mk_abort(a);
       return;

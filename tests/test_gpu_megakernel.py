@@ -139,6 +139,15 @@ def test_two_ragged_sequences_lossless_and_oracle():
     _check_first_step(w, W, P, max_seq_len=cap)
 
 
+def test_wide_model_lossless_and_oracle():
+    """d_model above 4096: the residual, norm and packing in separate passes
+    instead of one, more than one 1024-column chunk past a power of two."""
+    shape = tiny_shape(n_layers=4, d_model=4608, n_heads=36, n_kv_heads=9, head_dim=128, d_ffn=1408, vocab=4000)
+    w = _bf16_case().with_(shape=shape, gen_tokens=24)
+    W, P, _ = _lossless(w)
+    _check_first_step(w, W, P)
+
+
 @pytest.mark.parametrize("n", [62, 126, 127, 128, 640, 2100])
 def test_attention_ranges(n):
     """Contexts around the edges of the attention's position ranges (chunks of
