@@ -32,9 +32,9 @@
 // What bounds it: the tensor pipe.  At hd 128 a chunk's S takes 1280 cycles
 // and its P V 1700 (16 MMAs of 128 x 128 x 16 each; 1024 at the pipe's nominal
 // rate, which N = 128 does not reach), a softmax 1700; two tiles take 6200
-// cycles a chunk, 96 % of it MMA time.  1024 rows over 32 heads: 33 us (62 on
+// cycles a chunk, 96 % of it MMA time.  1024 rows over 32 heads: 40 us (62 on
 // warp MMAs, 64 vectors per CTA and chunks of 64 positions), over a cached
-// prefix of 8192 positions on average 232 us (834).
+// prefix of 8192 positions on average 228 us (834).
 //
 // Every wait is bounded (flag, then wind down).
 #include <algorithm>
@@ -77,7 +77,7 @@ __device__ __forceinline__ float ex2(float x) {
 template <int HD>
 __global__ void __launch_bounds__(kAfThreads, 1)
     attn_pf_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv,
-                   const __grid_constant__ AttnArgs a, int n_tiles, int fold) {
+                   const __grid_constant__ AttnArgs a, int n_tiles) {
   using SM = AfSmem<HD>;
   extern __shared__ uint8_t dsm_raw[];
   const uint32_t raw = smem_u32(dsm_raw);
@@ -97,13 +97,7 @@ __global__ void __launch_bounds__(kAfThreads, 1)
   const int g = blockIdx.x;
   const int grp = static_cast<int>(gridDim.y) - 1 - static_cast<int>(blockIdx.y);   // longest prefixes first
   const int sl = blockIdx.z, seq = a.seq0 + sl;
-  // first pass row of tile t; past the pass: no such tile
-  auto tile_row = [&](int t) {
-    if (!fold) return t < n_tiles ? (grp * n_tiles + t) * RT : a.rows_per_seq;
-    const int y = blockIdx.y, last = (a.rows_per_seq + RT - 1) / RT - 1;
-    if (t == 0) return y * RT;
-    return last - y > y ? (last - y) * RT : a.rows_per_seq;
-  };
+  const int i0 = grp * n_tiles * RT;                   // first pass row
 
   if (tid == 0) {
     for (int s = 0; s < kAfStages; ++s) {
@@ -133,7 +127,7 @@ __global__ void __launch_bounds__(kAfThreads, 1)
   const int base = a.lens[seq] + a.pos_off;            // position of pass row 0
   // chunks of tile t (0: the tile has no row)
   auto chunks = [&](int t) {
-    const int r0 = tile_row(t), nr = min(RT, a.rows_per_seq - r0);
+    const int r0 = i0 + t * RT, nr = t < n_tiles ? min(RT, a.rows_per_seq - r0) : 0;
     if (nr <= 0) return 0;
     return max(0, min(base + r0 + nr - 1, a.max_len - 1)) / kAfPos + 1;
   };
@@ -235,8 +229,8 @@ __global__ void __launch_bounds__(kAfThreads, 1)
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kAfSoftRegs));
     const int t = warp >> 2, wq = warp & 3;
-    const int r0 = tile_row(t);
-    const int nrows = max(0, min(RT, a.rows_per_seq - r0));
+    const int r0 = i0 + t * RT;
+    const int nrows = t < n_tiles ? max(0, min(RT, a.rows_per_seq - r0)) : 0;
     // ---------------- the tile's queries as hi / lo planes: a warp per vector,
     // four dims a lane
     {
@@ -388,15 +382,8 @@ cudaError_t launch_af(const AttnArgs& a, cudaStream_t s) {
   const long heads = static_cast<long>(a.n_kv_heads) * a.n_seqs;
   const long w1 = (heads * u1 + a.n_sms - 1) / a.n_sms, w2 = (heads * u2 + a.n_sms - 1) / a.n_sms;
   const int n_tiles = w1 * 4700 <= w2 * 6200 ? 1 : 2;
-  // Pairs that all run at once end with the longest one: then a CTA takes the
-  // pass's y-th tile and its y-th from the end, so the last tile's chunks are
-  // partly walked alone (the last two together: 8 chunks of 6200 cycles at
-  // 1024 rows; the first and the last: one, and seven of 4700; 38 -> 33 us
-  // over 32 heads, with a cached prefix of 8192 positions 238-246 -> 232).  In
-  // several waves the total counts, and neighbours share every chunk.
-  const int fold = n_tiles == 2 && heads * u2 <= a.n_sms ? 1 : 0;
   return launch_pdl(attn_pf_kernel<HD>, dim3(a.n_kv_heads, n_tiles == 1 ? u1 : u2, a.n_seqs), dim3(kAfThreads),
-                    AfSmem<HD>::kTotal, s, *a.kmap, *a.vmap, a, n_tiles, fold);
+                    AfSmem<HD>::kTotal, s, *a.kmap, *a.vmap, a, n_tiles);
 }
 }  // namespace
 
