@@ -316,8 +316,8 @@ dvi_status dvi_linear(dvi_ctx* ctx, const void* d_w, int n_out, int k_in,
  *  - The first call on a device looks up the scratch address for that
  *    device; make that first call before any stream capture.
  *  - All calls on a device share the one scratch array, and it keeps the
- *    last call's contents (split f32 calls clear its counters at their
- *    start, bf16 calls use none): calls that overlap on the GPU, e.g. on two streams, race. */
+ *    last call's contents (f32 calls whose splits meet there clear its
+ *    counters at their start, bf16 calls use none): calls that overlap on the GPU, e.g. on two streams, race. */
 dvi_status dvi_linear_noalloc(int dtype, const void* d_w, int n_out, int k_in, const float* d_x,
                               int m_rows, float* d_y, dvi_stream stream);
 

@@ -90,6 +90,7 @@ struct ProjMaps {
 // Picks n_splits / kb_per_split from the weight shape only (never from M),
 // so a row's result does not depend on how many rows share the launch.
 void plan_splits(ProjArgs& a, int n_sms, bool tc);
+bool proj_f32_cluster(const ProjArgs& a);
 size_t proj_partial_floats(const ProjArgs& a, bool tc);
 bool make_weight_map(CUtensorMap* map, const void* w, int rows, int cols);
 bool make_half_weight_map(CUtensorMap* map, const void* w, int rows, int cols);   // 64-row boxes (gate/up)

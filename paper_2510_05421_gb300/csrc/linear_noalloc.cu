@@ -116,9 +116,9 @@ extern "C" dvi_status dvi_linear_noalloc(int dtype, const void* d_w, int n_out, 
   if (tc && !make_weight_map(&maps.m0, d_w, n_out, k_in)) return DVI_ERR_INVALID_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   // A call that stopped early could leave counters raised; start from zero.
-  // Only splits that meet in global scratch count (f32): the bf16 kernel
-  // reduces inside its cluster, and the clearing would be a second launch.
-  if (!tc && a.n_splits > 1 && cudaMemsetAsync(s.counters, 0, sizeof(int) * n_counters, st) != cudaSuccess)
+  // Only splits that meet in global scratch count (f32): the others reduce
+  // inside their cluster, and the clearing would be a second launch.
+  if (!tc && a.n_splits > 1 && !proj_f32_cluster(a) && cudaMemsetAsync(s.counters, 0, sizeof(int) * n_counters, st) != cudaSuccess)
     return DVI_ERR_CUDA;
   if (launch_proj(a, tc ? &maps : nullptr, st) != cudaSuccess) return DVI_ERR_CUDA;
   return DVI_OK;

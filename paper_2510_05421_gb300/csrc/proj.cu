@@ -1147,8 +1147,13 @@ __global__ void __launch_bounds__(192, 2) proj_chain_kernel(const __grid_constan
 // flight while this one is multiplied, the first one issued before the wait
 // for the previous kernel (nothing earlier writes the weights).  NJ: token
 // columns computed, 4 for launches of at most four rows, else 16.
-// Tiny f32 decoder (d 256, 71 launches a step): 0.95 -> 0.42 ms a step.
-template <int NJ>
+// Tiny f32 decoder (d 256, 71 launches a step): 0.95 -> 0.42 ms a step
+// (0.38 with kCluster).
+// kCluster (proj_f32_cluster): the splits of a tile are a cluster that meets in
+// shared memory, rank r finishing its share of the token columns; else they
+// meet in global scratch and the last CTA finishes the tile.  Both add in
+// split order.
+template <int NJ, bool kCluster>
 __global__ void __launch_bounds__(128) proj_f32_kernel(const ProjArgs p) {
   __shared__ float Ws[kTileRows][kKBlockF32 + 1];
   __shared__ __align__(16) float Bs[kKBlockF32][kChunk];   // [k][token column]
@@ -1270,6 +1275,37 @@ __global__ void __launch_bounds__(128) proj_f32_kernel(const ProjArgs p) {
   float* rs = rstd - c0;
   const int* ps = posn - c0;
   float2 pre[kChunk];
+  if constexpr (kCluster) {
+    const int S = p.n_splits;
+    uint32_t mine = valid_cols(p, c0);
+#pragma unroll
+    for (int j = 0; j < kChunk; ++j)
+      if (j >= NJ || j < NJ * split / S || j >= NJ * (split + 1) / S) mine &= ~(1u << j);
+    float* part = &Ws[0][0];   // [NJ][128]: the weights have been used
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) part[j * kTileRows + row] = acc[j];
+    epi_pre<float>(p, tile, row, c0, mine, ps, pre);
+    cluster_arrive_release();
+    cluster_wait_acquire();
+    uint32_t peer[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) peer[r] = mapa_shared(smem_u32(part + row), r < S ? r : 0);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      acc[j] = 0.f;
+      if (!(mine >> j & 1u)) continue;
+      float t[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) t[r] = r < S ? ld_cluster_f32(peer[r] + j * kTileRows * 4) : 0.f;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < S) acc[j] += t[r];
+    }
+    cluster_arrive_release();   // this rank has read its peers' shared memory
+    if (mine) epilogue_chunk<float>(p, tile, row, c0, acc, pre, rs, ps, es, mine);
+    cluster_wait_acquire();
+    return;
+  }
   epi_pre<float>(p, tile, row, c0, valid_cols(p, c0), ps, pre);
   if (p.n_splits == 1) {
     epilogue_chunk<float>(p, tile, row, c0, acc, pre, rs, ps, es, valid_cols(p, c0));
@@ -1338,7 +1374,14 @@ void plan_splits(ProjArgs& a, int n_sms, bool tc) {
   a.kb_per_split = best_kbps;
 }
 
+// f32 launches whose splits meet in a cluster: of a portable size, and few
+// rows, where the exchange is a launch's latency (6.7 -> 5.5 us a launch of the
+// tiny decoder).  With more rows the CTAs come in waves, and a CTA that waits
+// for its cluster keeps the next one out: up to 11 % slower.
+bool proj_f32_cluster(const ProjArgs& a) { return a.n_splits > 1 && a.n_splits <= 8 && a.M <= 4; }
+
 // Global split-K scratch (f32 path only; bf16 reduces inside the cluster).
+// Sized for every split f32 launch, whether or not it meets in a cluster.
 size_t proj_partial_floats(const ProjArgs& a, bool tc) {
   if (tc || a.n_splits <= 1) return 0;
   const int ntt = (a.M + kChunk - 1) / kChunk;
@@ -1406,8 +1449,22 @@ cudaError_t launch_proj(const ProjArgs& a0, const ProjMaps* maps, cudaStream_t s
   } else {
     ProjArgs b = a0;
     b.n_ttiles = (a0.M + kChunk - 1) / kChunk;
-    e = launch_pdl(a0.M <= 4 ? proj_f32_kernel<4> : proj_f32_kernel<16>, dim3(a0.n_tiles * a0.n_splits, b.n_ttiles),
-                   dim3(128), 0, s, b);
+    const bool cl = proj_f32_cluster(b);
+    auto kern = cl ? proj_f32_kernel<4, true> : a0.M <= 4 ? proj_f32_kernel<4, false> : proj_f32_kernel<16, false>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a0.n_tiles * a0.n_splits, b.n_ttiles);
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = a0.n_splits;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cl ? 2 : 1;
+    e = cudaLaunchKernelEx(&cfg, kern, b);
   }
   return e != cudaSuccess ? e : cudaGetLastError();
 }
