@@ -33,9 +33,10 @@
 // each leaves its partial tile in shared memory and, after a cluster barrier,
 // rank r sums the partials of all ranks in rank order through distributed
 // shared memory for its contiguous share of the token columns and runs their
-// epilogue.  f32: each split stores its partial in
-// global scratch and the last CTA to arrive (an atomic counter per tile) sums
-// them in split order.  Both are deterministic, and the split plan depends on
+// epilogue.  f32: the same for up to four rows and eight splits; otherwise
+// each split stores its partial in global scratch and the last CTA to arrive
+// (an atomic counter per tile) sums them in split order.  Both are
+// deterministic, and the split plan depends on
 // the weight shape only (never on the number of decode rows).
 //
 // Persistent chain (bf16, opt-in): one launch runs several projections of
