@@ -289,7 +289,9 @@ dvi_status dvi_get_timing(dvi_ctx* ctx, double* ms, int* counts);
 /* Y[M][n_out] = X[M][K] . W[n_out][K]^T through the library's projection
  * kernel (tcgen05 for bf16, FP32 FMA for f32), with X float32 (for bf16
  * weights carried as a bf16 pair hi + lo, about 16 significant bits) and Y
- * float32, on the context's stream.  M <= 256.
+ * float32, on the context's stream.  M <= 256.  d_w and d_x may come from the
+ * work enqueued just before the call (another call's d_y, a trained W^(S)):
+ * neither is read before that is done.
  * A building block exposed for tests of the projection kernel itself. */
 dvi_status dvi_linear(dvi_ctx* ctx, const void* d_w, int n_out, int k_in,
                       const float* d_x, int m_rows, float* d_y);
@@ -315,9 +317,13 @@ dvi_status dvi_linear(dvi_ctx* ctx, const void* d_w, int n_out, int k_in,
  *    4096 x 4096 weight fits for up to 32 rows.
  *  - The first call on a device looks up the scratch address for that
  *    device; make that first call before any stream capture.
+ *  - d_w and d_x may come from the work enqueued on `stream` just before the
+ *    call (another call's d_y, a W^(S) that an update steps): neither is read
+ *    before that is done.
  *  - All calls on a device share the one scratch array, and it keeps the
  *    last call's contents (f32 calls whose splits meet there clear its
- *    counters at their start, bf16 calls use none): calls that overlap on the GPU, e.g. on two streams, race. */
+ *    counters at their start, bf16 calls use none): calls that overlap on
+ *    the GPU, e.g. on two streams, race. */
 dvi_status dvi_linear_noalloc(int dtype, const void* d_w, int n_out, int k_in, const float* d_x,
                               int m_rows, float* d_y, dvi_stream stream);
 

@@ -1638,6 +1638,7 @@ dvi_status dvi_linear(dvi_ctx* ctx, const void* d_w, int n_out, int k_in, const 
   Pass ps{nullptr, nullptr, 0, m_rows, 1, 0, 1, 0, nullptr, nullptr};
   ProjArgs a = base_args(ctx, EPI_HEAD, pl, ps);
   a.b_mode = B_SOFT_F32;
+  a.prefetch_a = 0;   // d_w may be the previous launch's output
   a.act = d_x;
   a.ld_act = k_in;
   a.K = k_in;

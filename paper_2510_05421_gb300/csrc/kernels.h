@@ -32,7 +32,10 @@ struct ProjArgs {
   int n_out;          // rows of one weight (GATEUP: F, tiles of 64 gate + 64 up rows); QKV uses rows_q/k/v
   int K;              // input features
   int n_tiles, n_splits, kb_total, kb_per_split, n_ttiles;
-  int prefetch_a;     // stream weight tiles before waiting for the previous kernel
+  // stream weight tiles before waiting for the previous kernel: only for weights
+  // that no earlier launch can still be writing (the frozen layers and LM head;
+  // neither a caller's own matrix nor a W^S that updates step)
+  int prefetch_a;
   const void* w0;     // f32 path: weight pointers (QKV: wq, wk, wv; GATEUP: gate, up)
   const void* w1;
   const void* w2;

@@ -94,7 +94,7 @@ extern "C" dvi_status dvi_linear_noalloc(int dtype, const void* d_w, int n_out, 
   a.n_ttiles = 1;
   a.rows_per_seq = 1;
   a.b_mode = B_SOFT_F32;
-  a.prefetch_a = 1;
+  a.prefetch_a = 0;   // d_w may be the previous launch's output
   a.act = d_x;
   a.ld_act = k_in;
   a.w0 = d_w;

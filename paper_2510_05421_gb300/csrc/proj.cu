@@ -1146,8 +1146,9 @@ __global__ void __launch_bounds__(192, 2) proj_chain_kernel(const __grid_constan
 // warp reads four whole 128-byte row pieces per instruction; single floats
 // where K or a pointer rules the float4 out), the next block's batch in
 // flight while this one is multiplied, the first one issued before the wait
-// for the previous kernel (nothing earlier writes the weights).  NJ: token
-// columns computed, 4 for launches of at most four rows, else 16.
+// for the previous kernel where prefetch_a allows it (weights that no earlier
+// launch writes).  NJ: token columns computed, 4 for launches of at most four
+// rows, else 16.
 // Tiny f32 decoder (d 256, 71 launches a step): 0.95 -> 0.42 ms a step
 // (0.38 with kCluster).
 // kCluster (proj_f32_cluster): the splits of a tile are a cluster that meets in
@@ -1219,8 +1220,9 @@ __global__ void __launch_bounds__(128) proj_f32_kernel(const ProjArgs p) {
       bv[e] = (n < p.M && kg < p.K) ? act[static_cast<size_t>(p.act_row0 + n) * p.ld_act + kg] : 0.f;
     }
   };
+  if (!p.prefetch_a) griddep_wait();
   if (nkb > 0) load_w(0);
-  griddep_wait();
+  griddep_wait();   // (at once the second time)
   if (nkb > 0) load_b(0);
   if (tid < kChunk) {
     float r = 1.f;

@@ -87,3 +87,79 @@ def test_f32_any_k_and_alignment(n, k, m, off):
     # K products and sums of f32: at most (K + 1) 2^-24 of sum |x||w|
     bound = (k + 1) * 2.0 ** -24 * (np.abs(X).astype(np.float64) @ np.abs(W).astype(np.float64).T)
     assert (np.abs(y.cpu().numpy() - ref) <= bound).all()
+
+
+# columns of the second weight and rows it is multiplied with: one K range;
+# ranges that meet in a cluster; in global scratch (more than four rows, more
+# than eight ranges)
+CHAINED = [(64, 4), (512, 4), (512, 16), (4096, 4)]
+
+
+@pytest.mark.parametrize("entry", ["noalloc", "context"])
+@pytest.mark.parametrize("k,m", CHAINED)
+def test_f32_weight_is_the_output_of_the_call_before(entry, k, m):
+    """y = x a^T (24 rows), then z = q y^T right behind it on the same stream: the second
+    call reads its weight only when the first is done.  Bit for bit the same
+    calls with a synchronisation between them; y is NaN before each pair."""
+    import ctypes
+    from paper_2510_05421_gb300.dvi import lib, linear_noalloc
+    g = torch.Generator(device="cuda")
+    g.manual_seed(k + m)
+    a = torch.randn(k, 2048, device="cuda", generator=g)
+    q = torch.randn(m, k, device="cuda", generator=g)
+    e, _, _ = engine_for(workload("tiny"), use_graphs=False)
+    torch.cuda.synchronize()
+
+    def linear(w, x, y):
+        if entry == "noalloc":
+            return linear_noalloc(w, x, y, stream=e.stream)
+        p = [ctypes.c_void_p(t.data_ptr()) for t in (w, x, y)]
+        return lib().dvi_linear(e.ctx, p[0], w.shape[0], w.shape[1], p[1], x.shape[0], p[2])
+
+    def pair(x, between):
+        y = torch.full((24, k), float("nan"), device="cuda")
+        z = torch.full((m, 24), float("nan"), device="cuda")
+        torch.cuda.synchronize()
+        assert linear(a, x, y) == 0
+        between()
+        assert linear(y, q, z) == 0
+        torch.cuda.synchronize()
+        return y, z
+
+    for _ in range(10):
+        x = torch.randn(24, 2048, device="cuda", generator=g)
+        y1, z1 = pair(x, lambda: None)
+        y2, z2 = pair(x, torch.cuda.synchronize)
+        assert torch.equal(y1, y2) and torch.equal(z1, z2)
+    assert e.stats()["device_status"] == 0
+    e.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_projection_right_behind_the_update_that_steps_its_weight(dtype):
+    """linear_noalloc on W^S right behind a full-head update on the engine's
+    stream multiplies the stepped W^S (bit for bit the call after a
+    synchronisation), which the step has moved."""
+    from dataclasses import replace
+    from workloads import make_prompts
+    from paper_2510_05421_gb300.dvi import linear_noalloc
+    w = workload("tiny")
+    w = w.with_(shape=replace(w.shape, d_model=512, vocab=8192), dtype=dtype, update_every=4)
+    e, _, dw = engine_for(w, head_mode=1)
+    P = make_prompts(w)
+    u = torch.randn(4, 512, device="cuda")
+    y1, y2, old = (torch.full((4, 8192), float("nan"), device="cuda") for _ in range(3))
+    torch.cuda.synchronize()
+    for _ in range(3):
+        e.generate(P, 10 ** 6, max_steps=w.update_every, log=True)
+        assert linear_noalloc(dw.draft_head, u, old, stream=e.stream) == 0
+        e.sync()
+        e.update(w.update)
+        assert linear_noalloc(dw.draft_head, u, y1, stream=e.stream) == 0
+        e.sync()
+        assert linear_noalloc(dw.draft_head, u, y2, stream=e.stream) == 0
+        e.sync()
+        assert torch.equal(y1, y2)
+        assert not torch.equal(y1, old)
+    assert e.stats()["device_status"] == 0
+    e.close()
