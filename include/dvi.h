@@ -148,7 +148,10 @@ typedef struct {
  * lora_a / lora_b are updated in place by dvi_update_drafter (head_mode 0);
  * draft_head is updated in place in head_mode 1: with dtype bf16 the
  * optimizer steps an f32 master copy (taken from draft_head by dvi_create)
- * and writes its bf16 rounding back to draft_head after every update. */
+ * and writes its bf16 rounding back to draft_head after every update.
+ * Everything else is frozen, and its first tiles may be read ahead of the
+ * kernels that precede a call on the stream: what writes it must be complete
+ * before dvi_create. */
 typedef struct {
   const void* embed;              /* [V][d] */
   const dvi_layer_weights* layers;/* host array of L entries */

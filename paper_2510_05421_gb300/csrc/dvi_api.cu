@@ -897,6 +897,7 @@ dvi_status enqueue_head(dvi_ctx* ctx, bool draft, int rows, int logits_mode, con
   a.K = ctx->d;
   a.n_out = ctx->V;
   a.w0 = draft ? ctx->w.draft_head : ctx->w.lm_head;
+  if (draft && ctx->rt.head_mode == 1) a.prefetch_a = 0;   // an update steps W^S
   a.amax = ctx->amax;
   if (draft && ctx->r > 0) {
     a.lora_a = ctx->w.lora_a;
@@ -1457,6 +1458,7 @@ dvi_status dvi_update_drafter(dvi_ctx* ctx, const dvi_update_config* u) {
   p.K = ctx->d;
   p.n_out = ctx->V;
   p.w0 = ctx->w.draft_head;
+  if (full) p.prefetch_a = 0;   // the update before steps W^S
   p.logits_mode = 1;
   p.logits_out = ctx->Z;
   p.ld_logits = ctx->V;

@@ -1192,8 +1192,9 @@ __global__ void update_master_init_kernel(const __nv_bfloat16* w, float* master,
     master[i] = __bfloat162float(w[i]);
 }
 
+// Ends a full-head update.  It does not let its dependents start early: what
+// follows an update may read W^S, and starts after every CTA that steps it.
 __global__ void update_finish_kernel(const UpdateArgs a) {
-  griddep_launch();
   griddep_wait();
   finish_body(a, threadIdx.x, blockDim.x);
 }

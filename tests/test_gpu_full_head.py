@@ -125,6 +125,28 @@ def test_bf16_full_head_lossless_and_gradient():
     assert torch.equal(torch.from_numpy(w_new).bfloat16().float(), torch.from_numpy(w_new))
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_eager_steps_read_the_stepped_head(dtype):
+    """Eager launches (no graph between an update and the next draft: one chain
+    of early launches) against graph replays, with the per-kernel draft path:
+    tokens, accept lengths and the trained W^S bit for bit."""
+    w = workload("tiny").with_(dtype=dtype, update_every=2)
+    w = w.with_(shape=replace(w.shape, n_layers=2, vocab=8192), split_k=1)
+    W = make_weights(w)
+    P = make_prompts(w)
+    outs = []
+    for graphs in (True, False):
+        eng, _, dw = engine_for(w, W=W, head_mode=1, use_graphs=graphs, megakernel=False)
+        toks, mats, _, _ = eng.generate(P, w.gen_tokens, update_every=2, hyper=w.update)
+        st = eng.stats()
+        assert st["device_status"] == 0 and st["updates"] >= 4
+        outs.append((toks, mats, dw.draft_head.clone()))
+        eng.close()
+    assert outs[0][0] == outs[1][0]
+    assert np.array_equal(outs[0][1], outs[1][1])
+    assert torch.equal(outs[0][2], outs[1][2])
+
+
 @pytest.mark.parametrize("steps,vocab", [(7, 1021), (8, 1024), (12, 1021)])
 def test_gradient_tiles(steps, vocab):
     """dL/dW^(S) and the step by both kernels: U kept in shared memory (buffers
