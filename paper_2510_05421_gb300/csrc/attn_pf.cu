@@ -133,6 +133,11 @@ __global__ void __launch_bounds__(kAfThreads, 1)
   };
   const int nch0 = chunks(0), nch1 = chunks(1);
   const int nch = max(nch0, nch1);
+  // Rows of the last chunk from here on lie past every position that the CTA's
+  // rows see: an earlier request's, another head's, or never written.  The
+  // probability 0 of such a row leaves NaN in O if its value is not finite, so
+  // the values there are cleared in shared memory.
+  const int past = min(base + min(i0 + n_tiles * RT, a.rows_per_seq) - 1, a.max_len - 1) % kAfPos + 1;
 
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kAfOtherRegs));
@@ -269,6 +274,23 @@ __global__ void __launch_bounds__(kAfThreads, 1)
     bool ok = true;
 #pragma unroll 1
     for (int i = 0; i < my; ++i) {
+      // the first tile that has the last chunk clears its values past the end
+      // before its probabilities let P V start.  (The stage's copy before this
+      // one, K chunk i - 1, is complete: its scores were read; none follows.)
+      if (i == nch - 1 && t == (nch0 == nch ? 0 : 1) && past < kAfPos) {
+        const int iv = 2 * i + 1, sv = iv % kAfStages;
+        if (!mbar_wait(&full[sv], (iv / kAfStages) & 1, a.status)) {
+          ok = false;
+          break;
+        }
+        uint8_t* vs = sm + SM::kRing + sv * SM::kStage;
+        for (int e = wq * 32 + lane; e < (kAfPos - past) * (HD / 8); e += kAfQ) {
+          const int row = past + e / (HD / 8), q = e % (HD / 8);
+          *reinterpret_cast<uint4*>(vs + (q >> 3) * SM::kBox + sw128_offset(row, 8 * (q & 7))) =
+              make_uint4(0u, 0u, 0u, 0u);
+        }
+        fence_proxy_async_smem();
+      }
       if (!mbar_wait(&s_full[t], i & 1, a.status)) {
         ok = false;
         break;

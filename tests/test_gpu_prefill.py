@@ -143,3 +143,39 @@ def test_short_prompts_split_over_k(d, hq, hkv, hd, f, n):
             assert np.abs(got[l] - r).max() <= 2.0 ** -7 * np.abs(r).max(), l
     k2, v2, first2 = _prefill(w, dw, P, 48)
     assert np.array_equal(k, k2) and np.array_equal(v, v2) and first == first2
+
+
+# (query heads, KV heads, head_dim, prompt): the last chunk of 128 positions
+# nearly empty and nearly full, two tiles of a CTA that end in different chunks,
+# a full last chunk
+STALE = [(4, 4, 64, 1), (4, 2, 128, 127), (16, 2, 64, 130), (32, 32, 64, 700), (20, 20, 128, 1025), (4, 4, 64, 256)]
+
+
+@pytest.mark.parametrize("hq,hkv,hd,n", STALE)
+def test_values_behind_the_prompt_do_not_matter(hq, hkv, hd, n):
+    """A cache whose other rows (an earlier request's, the neighbouring heads'
+    and sequences') are NaN: the prompt's K/V rows and first token are bit for
+    bit those of a clean cache."""
+    from paper_2510_05421_gb300 import DVIEngine, DeviceWeights
+    from workloads import tiny_shape
+    w = workload("tiny").with_(dtype="bf16", prompt_len=(n, n), split_k=1,
+                               shape=tiny_shape(n_layers=2, n_heads=hq, n_kv_heads=hkv, head_dim=hd))
+    dw = DeviceWeights.from_host(make_weights(w), "bf16")
+    prompt = torch.from_numpy(make_prompts(w)[0]).cuda()
+    room = n + 9
+    outs = []
+    for stale in (0.0, float("nan")):
+        eng = DVIEngine(w.shape, "bf16", dw, batch=2, k_spec=w.k_spec, split_k=1, lora_rank=w.lora_rank,
+                        lora_gamma=w.lora_gamma, max_seq_len=room, log_steps=1)
+        rows = [eng.buffer(b, torch.bfloat16) for b in ("K_CACHE", "V_CACHE")]
+        for r in rows:
+            r.fill_(stale)
+        torch.cuda.synchronize()
+        eng.prefill(0, prompt)
+        eng.sync()
+        assert eng.stats()["device_status"] == 0
+        outs.append([r.view(2, 2, hkv, room, hd)[:, 0, :, :n].clone() for r in rows] + [int(eng.first[0])])
+        eng.close()
+    assert all(torch.isfinite(t).all() for t in outs[1][:2])
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    assert outs[0][2] == outs[1][2]
