@@ -477,6 +477,16 @@ __global__ void __launch_bounds__(128) attn_mma_kernel(const __grid_constant__ C
     const uint8_t* ks = ring + st * kStage;
     const uint8_t* vs = ks + kBoxes * kBoxBytes;
     const int pc = (c0 + ch) * kChunkPos;
+    // V rows past the last position that any row of the CTA sees (an earlier
+    // request's, another head's) are cleared in the stage, the CTA's last: 0
+    // times a value that is not finite is NaN.
+    if (pc + kChunkPos - 1 > p_max) {
+      constexpr int kPer = 256 / HD;   // rows a warp clears at a time
+      for (int i = p_max + 1 - pc + warp * kPer + lane / (HD / 8); i < kChunkPos; i += 4 * kPer)
+        *reinterpret_cast<uint4*>(const_cast<uint8_t*>(vs) + ((lane % (HD / 8)) >> 3) * kBoxBytes +
+                                  sw128_offset(i, 8 * (lane & 7))) = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
+    }
     // S = Q K^T for this warp's 16 positions (two n-tiles of 8)
     float sacc[2][4], slo[2][4];   // q_hi K^T and q_lo K^T: independent MMA chains
 #pragma unroll

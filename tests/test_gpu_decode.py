@@ -210,3 +210,36 @@ def test_drafter_head_lora_blocks(batch, rank):
     ws = rounded_weights(W).draft_head.astype(np.float64)
     ref = u @ ws.T + (u @ W.lora_b.astype(np.float64).T) @ W.lora_a.astype(np.float64).T
     assert np.abs(z - ref).max() <= 1e-4 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("dtype,megakernel", [("bf16", True), ("bf16", False), ("f32", False)])
+def test_rows_behind_the_sequence_do_not_matter(dtype, megakernel):
+    """Decoding in a cache whose unwritten rows are NaN (an earlier request's
+    leftovers, behind each sequence and in front of the next head's) gives the
+    tokens, accept lengths and K/V rows of a clean cache bit for bit."""
+    w = (_bf16_case() if dtype == "bf16" else workload("tiny")).with_(batch=2, prompt_len=(37, 90), gen_tokens=24)
+    W = make_weights(w)
+    P = make_prompts(w)
+    td = torch.bfloat16 if dtype == "bf16" else torch.float32
+    outs = []
+    for stale in (0.0, float("nan")):
+        for ar in (False, True):
+            eng, _, _ = engine_for(w, W=W, megakernel=megakernel, max_seq_len=231)
+            rows = [eng.buffer(b, td) for b in ("K_CACHE", "V_CACHE")]
+            for r in rows:
+                r.fill_(stale)
+            torch.cuda.synchronize()
+            if ar:
+                got = eng.generate_ar(P, w.gen_tokens).tolist()
+            else:
+                toks, mats, _, _ = eng.generate(P, w.gen_tokens)
+                got = [toks, mats.tolist()]
+            st = eng.stats()
+            assert st["device_status"] == 0, st["device_flags"]
+            n = eng.buffer("LENS", torch.int32).tolist()
+            kv = [r.view(w.shape.n_layers, 2, w.shape.n_kv_heads, 231, w.shape.head_dim) for r in rows]
+            outs.append((got, n, [r[:, b, :, :n[b]].clone() for r in kv for b in range(2)]))
+            eng.close()
+    for a, b in ((0, 2), (1, 3)):
+        assert outs[a][:2] == outs[b][:2]
+        assert all(torch.equal(x, y) for x, y in zip(outs[a][2], outs[b][2]))
