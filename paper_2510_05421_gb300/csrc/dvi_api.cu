@@ -61,6 +61,7 @@ struct dvi_ctx {
   std::vector<dvi_layer_weights> layers;
   cudaStream_t stream = nullptr;
   int n_sms = 152;
+  int dev = 0;   // the workspace's GPU
   bool tc = false;
   size_t esz = 4;
   int L, d, Hq, Hkv, hd, F, V, k, r, B, K, max_len, cap_steps, cap_rows, chunk, M_max, nq, nkv;
@@ -103,7 +104,7 @@ struct dvi_ctx {
   bool mk_on = false;
   MkArgs mk{};
   size_t mk_sync_bytes = 0;
-  void* mk_sync = nullptr;   // argmax keys, then the completion counters and abort flag
+  void* mk_sync = nullptr;   // argmax keys, tagged words, then the completion counters and abort flag
   CUtensorMap* mk_maps_dev = nullptr;   // the kernel's weight descriptors (workspace)
   std::vector<CUtensorMap> mk_maps;     // their host copy (source of the upload)
   float* chain_part = nullptr;
@@ -1097,6 +1098,17 @@ void fill_rope_host(int max_len, int hd, float theta, std::vector<float2>& out) 
     }
 }
 
+// Whether a kernel on the context's GPU may store int32 values at p.
+bool storable_i32(const dvi_ctx* c, const void* p) {
+  if ((reinterpret_cast<uintptr_t>(p) & 3u) != 0) return false;
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == c->dev;
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 cudaEvent_t take_event(dvi_ctx* c) {
@@ -1210,6 +1222,9 @@ dvi_status dvi_create(const dvi_model_config* cfg, const dvi_runtime_config* rt,
     return DVI_ERR_CAPACITY;
   }
   ctx->ws = workspace;
+  cudaPointerAttributes ws_at{};
+  if (cudaPointerGetAttributes(&ws_at, workspace) == cudaSuccess) ctx->dev = ws_at.device;
+  else cudaGetLastError();
   layout(ctx, static_cast<char*>(workspace));
   ctx->w = *weights;
   ctx->layers.assign(weights->layers, weights->layers + cfg->n_layers);
@@ -1376,9 +1391,26 @@ dvi_status dvi_draft_verify_commit(dvi_ctx* ctx, int32_t* d_out_ids, int32_t* d_
   rc = run_graph(ctx, &ctx->verify_exec, &ctx->verify_launches, g, [&] { return enqueue_verify(ctx); });
   if (rc != DVI_OK) return rc;
   mark_end(ctx, 1, t1);
-  if (d_out_ids || d_n_committed || d_n_accepted) {
+  // one launch for the three where a kernel may write them all; copies, with
+  // the driver's checks, for anything else (another GPU's memory, an odd address)
+  struct Out {
+    int32_t* to;
+    const int* from;
+    int n;
+  } out[3] = {{d_out_ids, ctx->out_ids, ctx->B * ctx->Kv},
+              {d_n_committed, ctx->n_committed, ctx->B},
+              {d_n_accepted, ctx->n_accepted, ctx->B}};
+  bool any = false, direct = true;
+  for (const Out& o : out) {
+    any = any || o.to;
+    direct = direct && (!o.to || storable_i32(ctx, o.to));
+  }
+  if (any && direct) {
     DVI_CUDA(launch_copy_out(step_state(ctx), d_out_ids, d_n_committed, d_n_accepted, s));
     ctx->launches += 1;
+  } else {
+    for (const Out& o : out)
+      if (o.to) DVI_CUDA(cudaMemcpyAsync(o.to, o.from, sizeof(int) * o.n, cudaMemcpyDeviceToDevice, s));
   }
   return DVI_OK;
 }

@@ -243,3 +243,38 @@ def test_rows_behind_the_sequence_do_not_matter(dtype, megakernel):
     for a, b in ((0, 2), (1, 3)):
         assert outs[a][:2] == outs[b][:2]
         assert all(torch.equal(x, y) for x, y in zip(outs[a][2], outs[b][2]))
+
+
+@pytest.mark.parametrize("where", ["device", "odd", "null"])
+def test_step_outputs_at_any_address(where):
+    """The step's output buffers of the C call: plain device memory (one
+    kernel), addresses that an int32 store may not have (copies), and null."""
+    import ctypes
+    from paper_2510_05421_gb300.dvi import lib
+    w = workload("tiny")
+    P = make_prompts(w)
+    eng, W, _ = engine_for(w)
+    ref, _, _ = engine_for(w, W=W)
+    mem = torch.full((256,), 0x77, dtype=torch.uint8, device="cuda")
+    at = [mem.data_ptr() + 64 * i + (2 if where == "odd" else 0) for i in range(3)]
+    if where == "null":
+        at[1] = None
+    torch.cuda.synchronize()
+    prompt = torch.from_numpy(np.ascontiguousarray(P[0], dtype=np.int32)).cuda()
+    for e in (eng, ref):
+        e.prefill(0, prompt)
+    for _ in range(3):
+        assert lib().dvi_draft_verify_commit(eng.ctx, *[ctypes.c_void_p(p) for p in at]) == 0
+        want = ref.step()
+        eng.sync()
+        ref.sync()
+        host = mem.cpu().numpy().tobytes()
+        for i, t in enumerate(want):
+            if at[i] is None:
+                continue
+            o = at[i] - mem.data_ptr()
+            b = t.cpu().numpy().tobytes()
+            assert host[o:o + len(b)] == b
+            assert host[o + len(b):64 * (i + 1)] == b"\x77" * (64 * (i + 1) - o - len(b))
+    eng.close()
+    ref.close()
