@@ -386,17 +386,21 @@ __global__ void __launch_bounds__(kAfThreads, 1)
 }
 
 namespace {
+// Registers per thread that the kernel was compiled with.
+template <int HD>
+int af_regs() {
+  cudaFuncAttributes fa{};
+  if (cudaFuncGetAttributes(&fa, attn_pf_kernel<HD>) == cudaSuccess) return fa.numRegs;
+  cudaGetLastError();
+  return 0;
+}
+
 template <int HD>
 cudaError_t launch_af(const AttnArgs& a, cudaStream_t s) {
   static PerDevice attr;
-  static int regs = 0;
   attr.once([] {
     cudaFuncSetAttribute(attn_pf_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, AfSmem<HD>::kTotal);
-    cudaFuncAttributes fa{};
-    regs = cudaFuncGetAttributes(&fa, attn_pf_kernel<HD>) == cudaSuccess ? fa.numRegs : 0;
   });
-  // the softmax warps' register increase draws on what the block was launched with
-  if (regs * kAfThreads < 256 * kAfSoftRegs + 128 * kAfOtherRegs) return cudaErrorInvalidConfiguration;
   // One tile per CTA while the waves allow it: a lone tile's chunk is S,
   // softmax and P V in turn (about 4700 cycles at hd 128), a pair's 6200.
   const int rt = kAfQ / (a.n_heads / a.n_kv_heads);
@@ -408,6 +412,13 @@ cudaError_t launch_af(const AttnArgs& a, cudaStream_t s) {
                     AfSmem<HD>::kTotal, s, *a.kmap, *a.vmap, a, n_tiles);
 }
 }  // namespace
+
+// The softmax warps' register increase draws on what the block was launched
+// with and waits for ever if that is less than the split needs.
+bool attn_pf_ok(int head_dim) {
+  const int regs = head_dim == 128 ? af_regs<128>() : af_regs<64>();
+  return regs * kAfThreads >= 256 * kAfSoftRegs + 128 * kAfOtherRegs;
+}
 
 cudaError_t launch_attn_pf(const AttnArgs& a, cudaStream_t s) {
   return a.head_dim == 128 ? launch_af<128>(a, s) : launch_af<64>(a, s);

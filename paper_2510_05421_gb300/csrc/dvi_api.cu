@@ -1314,6 +1314,11 @@ dvi_status dvi_create(const dvi_model_config* cfg, const dvi_runtime_config* rt,
       return DVI_ERR_INVALID_ARG;
     }
   }
+  if (ctx->tc && ctx->Hq / ctx->Hkv <= 8 && !attn_pf_ok(ctx->hd)) {
+    fprintf(stderr, "dvi_create: the prompt attention kernel was compiled with too few registers a thread\n");
+    delete ctx;
+    return DVI_ERR_CUDA;
+  }
   std::vector<float2> rope;
   fill_rope_host(ctx->max_len, ctx->hd, cfg->rope_theta, rope);
   if (cudaMemsetAsync(workspace, 0, ctx->ws_bytes, ctx->stream) != cudaSuccess ||

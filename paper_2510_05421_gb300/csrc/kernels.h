@@ -173,7 +173,10 @@ bool make_kv_map(CUtensorMap* map, const void* cache, long long rows, int hd);
 size_t attn_partial_floats(const AttnArgs& a);
 int attn_counters(const AttnArgs& a);
 cudaError_t launch_attn(const AttnArgs& a, cudaStream_t s);
-// The prefill attention kernel (attn_pf.cu; a.prefill set).
+// The prefill attention kernel (attn_pf.cu; a.prefill set), and whether the
+// compiled kernel has the registers that its warps share out (dvi_create
+// refuses a context that would launch it otherwise).
+bool attn_pf_ok(int head_dim);
 cudaError_t launch_attn_pf(const AttnArgs& a, cudaStream_t s);
 
 // ---- small kernels (misc.cu)
