@@ -208,8 +208,7 @@ def linear_noalloc(w: torch.Tensor, x: torch.Tensor, y: torch.Tensor, stream=Non
 
 
 def _linear_noalloc(w, x, y, dev: int, stream) -> int:
-    # the raw handle of torch's current stream, without a Stream object around it
-    s = torch._C._cuda_getCurrentRawStream(dev) if stream is None else stream.cuda_stream
+    s = (torch.cuda.current_stream(dev) if stream is None else stream).cuda_stream
     m, k = x.shape
     return lib().dvi_linear_noalloc(DVI_BF16 if w.dtype == torch.bfloat16 else DVI_F32, w.data_ptr(), w.shape[0], k,
                                     x.data_ptr(), m, y.data_ptr(), s)
