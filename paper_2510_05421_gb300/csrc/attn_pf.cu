@@ -29,12 +29,13 @@
 // other.  Shared memory: the queries (hi and lo of both tiles, 128 KB at hd
 // 128) and three 128-position K or V stages of 32 KB.
 //
-// What bounds it: the tensor pipe.  At hd 128 a chunk's S takes 1280 cycles
-// and its P V 1700 (16 MMAs of 128 x 128 x 16 each; 1024 at the pipe's nominal
-// rate, which N = 128 does not reach), a softmax 1700; two tiles take 6200
-// cycles a chunk, 96 % of it MMA time.  1024 rows over 32 heads: 40 us (62 on
-// warp MMAs, 64 vectors per CTA and chunks of 64 positions), over a cached
-// prefix of 8192 positions on average 228 us (834).
+// What bounds it: the MMAs at M = N = 128.  At hd 128 a chunk's S takes 1280
+// cycles and its P V 1700 (16 MMAs of 128 x 128 x 16 each, 80 to 105 cycles
+// apiece; 64, so 1024 for the 16, at the pipe's nominal rate), a softmax 1700.
+// Two tiles take 6200 cycles a chunk: an MMA is in flight in 96 % of them, but
+// by the nominal rate the pipe is two thirds busy (4096 cycles).  1024 rows
+// over 32 heads: 38.5 us (62 on warp MMAs, 64 vectors per CTA and chunks of 64
+// positions), over a cached prefix of 8192 positions on average 230 us (834).
 //
 // Every wait is bounded (flag, then wind down).
 #include <algorithm>
@@ -403,6 +404,11 @@ cudaError_t launch_af(const AttnArgs& a, cudaStream_t s) {
   });
   // One tile per CTA while the waves allow it: a lone tile's chunk is S,
   // softmax and P V in turn (about 4700 cycles at hd 128), a pair's 6200.
+  // At hd 64 the ratio serves too (32 heads, pairs against single tiles: 512
+  // rows 23.1 / 21.1 us, 2048 rows 88.5 / 96.0, 8192 rows 909 / 1192; 16 heads
+  // over 4 KV heads, always single here: 23.7 / 20.2, 95 / 77, 939 / 723) but
+  // where a pair saves the second of two waves (700 rows 29.6 / 25.9, 1024 rows
+  // 32.6 / 31.1: pairs are taken).
   const int rt = kAfQ / (a.n_heads / a.n_kv_heads);
   const int u1 = (a.rows_per_seq + rt - 1) / rt, u2 = (u1 + 1) / 2;
   const long heads = static_cast<long>(a.n_kv_heads) * a.n_seqs;

@@ -762,9 +762,6 @@ bool use_chain(const dvi_ctx* ctx, const Pass& ps) {
   return ctx->tc && !ps.pf && ctx->chain_ctas > 0 && (ps.M + 15) / 16 * 16 <= kChainMaxPad;
 }
 
-// One decoder layer on the pass's rows, one kernel per projection.  `g_last`
-// is the gain of whatever consumes the pass's residual after this layer (the
-// next layer's attention norm, or the final norm before a head).
 // A projection of a bf16 prompt pass on the prefill kernel, with the
 // activation buffer's 128-row map and the weights' 128-row maps.
 dvi_status run_proj_pf(dvi_ctx* ctx, const ProjLaunch& pl, int n_tokens, const CUtensorMap& act, const CUtensorMap& w0,
@@ -782,8 +779,8 @@ dvi_status run_proj_pf(dvi_ctx* ctx, const ProjLaunch& pl, int n_tokens, const C
   return DVI_OK;
 }
 
-// One layer of a bf16 prompt pass: QKV, gate/up, O and down on the prefill
-// kernel, the attention on the decode attention kernel.
+// One layer of a bf16 prompt pass on the prefill projection kernels and the
+// prefill attention kernel (GQA groups above 8: attn_smem_kernel).
 dvi_status enqueue_layer_pf(dvi_ctx* ctx, int l, const Pass& ps, const float* g_last) {
   const LayerMaps& m = ctx->maps[l];
   dvi_status st;
@@ -796,6 +793,9 @@ dvi_status enqueue_layer_pf(dvi_ctx* ctx, int l, const Pass& ps, const float* g_
   return run_proj_pf(ctx, down_launch(ctx, l, ps, g_last), ps.n_tokens, ctx->map_pf_ffn_h, m.down.m0);
 }
 
+// One decoder layer on the pass's rows, one kernel per projection.  `g_last`
+// is the gain of whatever consumes the pass's residual after this layer (the
+// next layer's attention norm, or the final norm before a head).
 dvi_status enqueue_layer(dvi_ctx* ctx, int l, const Pass& ps, const float* g_last) {
   if (ps.pf) return enqueue_layer_pf(ctx, l, ps, g_last);
   dvi_status st;

@@ -43,10 +43,11 @@ struct FinSmem {
 // One residual row from the embedding table (128 threads): x, x * g and the
 // per-tile sums of squares.  All of the row's loads are issued before any is
 // used (one memory round trip), then a single block barrier.
-template <typename T, int NT = kMaxTiles>
+template <typename T>
 __device__ void embed_row_block(const T* table, int tok, int d, float* x, const float* g, T* xg, size_t plane,
                                 float* ss, int ss_ld, int row, float* red) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NT = kMaxTiles;
   const int nt = d / kTileRows;
   const T* src = table + static_cast<size_t>(tok) * d;
   float v[NT], gv[NT];
@@ -291,7 +292,7 @@ __device__ void finalize_draft_body(const StepState& st, int j, const HeadPrepAr
 
 // Accept length, commit and rollback, the replay-buffer tuples' metadata,
 // and the next pass's embedding (finalize_verify).
-template <typename T, int NT = kMaxTiles>
+template <typename T>
 __device__ void finalize_verify_body(const StepState& st, FinSmem& fs) {
   const int K = st.K, Kv = st.Kv;
   // one round trip: every row's argmax and every drafted token by a thread of
@@ -347,7 +348,7 @@ __device__ void finalize_verify_body(const StepState& st, FinSmem& fs) {
 }
 
 // Greedy AR: the argmax is the next token of every sequence (finalize_ar).
-template <typename T, int NT = kMaxTiles>
+template <typename T>
 __device__ void finalize_ar_body(const StepState& st, FinSmem& fs) {
   for (int b = threadIdx.x; b < st.B; b += kFinThreads) {
     const int y = take_argmax(st.amax + b, st.status);
@@ -392,8 +393,8 @@ __device__ __forceinline__ void head_finalize(const FinArgs& f, uint8_t* smem, i
   uint8_t* emb = f.stage ? smem + (sizeof(FinSmem) + 15) / 16 * 16 : nullptr;
   // (the preparation ran in the head's first CTAs)
   if (f.kind == FIN_DRAFT) finalize_draft_body<__nv_bfloat16, NT>(f.st, f.j, f.hp, 0, fs, emb);
-  else if (f.kind == FIN_VERIFY) finalize_verify_body<__nv_bfloat16, NT>(f.st, fs);
-  else finalize_ar_body<__nv_bfloat16, NT>(f.st, fs);
+  else if (f.kind == FIN_VERIFY) finalize_verify_body<__nv_bfloat16>(f.st, fs);
+  else finalize_ar_body<__nv_bfloat16>(f.st, fs);
 }
 
 }  // namespace dvi

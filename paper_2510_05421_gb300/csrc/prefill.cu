@@ -195,11 +195,6 @@ __device__ __forceinline__ void pf_epi_qkv(const ProjArgs& p, uint32_t acc, int 
   }
 }
 
-// O and down: x += y, the next norm's activation rows x * g (hi/lo), and
-// the sums of squares of the new x per 128 features (in feature order).
-// The tile's residual row is read kResAhead steps of 16 features ahead of
-// its use (a step's four loads take about a microsecond, with one thread a
-// row and nothing else in flight: 16 of them in turn were a tail of 12 us).
 // A row's sum of squares over 128 features, added in one order everywhere:
 // four features at a time, then the tree of a warp that holds four a lane.
 __device__ __forceinline__ float sq4(float4 x) { return fmaf(x.w, x.w, fmaf(x.z, x.z, fmaf(x.y, x.y, x.x * x.x))); }
@@ -236,6 +231,11 @@ __device__ __forceinline__ void pf_put_resid(const ProjArgs& p, int n, int f, co
     st_act16(static_cast<__nv_bfloat16*>(p.xg_out) + static_cast<size_t>(n) * p.ld_xg + f, p.xg_plane, y);
   }
 }
+// O and down: x += y, the next norm's activation rows x * g (hi/lo), and
+// the sums of squares of the new x per 128 features (in feature order).
+// The tile's residual row is read kResAhead steps of 16 features ahead of
+// its use (a step's four loads take about a microsecond, with one thread a
+// row and nothing else in flight: 16 of them in turn were a tail of 12 us).
 __device__ __forceinline__ void pf_epi_resid(const ProjArgs& p, uint32_t acc, int nt, int h, int n, bool live,
                                              Ahead& ahead) {
   const int f0 = nt * kPfN + h * kTileRows;
@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(kPsThreads, 1)
     cluster_wait_acquire();
   }
   if (warp < kPsEpi && ok) {
-    // ---------------- epilogue: row i of the rank by warp i mod 8
+    // ---------------- epilogue: row i of the rank by warp i mod kPsEpi
     const uint32_t mine = smem_u32(part);
     const int rows = min(R, p.M - n0);
     if (p.flavor == EPI_QKV) {
